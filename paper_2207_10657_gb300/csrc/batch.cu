@@ -29,6 +29,7 @@ using R = float;
 using C = float2;
 
 constexpr int kMaxBatch = 256;
+constexpr int kXYPerSM = 8;               // blocks per SM of the x / y / 2D launches
 constexpr long long kVecChunk = 16384;  // field elements per vector item (multiple of 4)
 constexpr long long kVoxChunk = 4096;   // voxels per constitutive item (multiple of 4)
 
@@ -38,10 +39,9 @@ struct BDesc {
   GridDesc g;
   AxisPlan px, py, pz;
   const C* tw[3];
-  const C* gd[3];
-  const C* ga[3];
+  AxisSyms<R> sy;
   C* spec;
-  int qx, ty, tz;
+  int qx, lty, ltz;
   unsigned free_mask;
   long long foff;  // first field element of this RVE in the batched vectors
   long long voff;  // first voxel of this RVE in the batched scalar fields
@@ -118,22 +118,33 @@ __global__ void kb_compact(WLists* wl, const int* __restrict__ nb, int n, Gate g
   }
 }
 
+// The item's member descriptor, copied to shared memory: the stage loops
+// read the plan's fields over and over.  (fetch() has synchronised since the
+// block's last use of the copy.)
+__device__ __forceinline__ const BDesc& member_desc(const BDesc* d, int* s) {
+  static_assert(sizeof(BDesc) % 4 == 0, "copied as words");
+  for (int i = threadIdx.x; i < (int)(sizeof(BDesc) / 4); i += blockDim.x) s[i] = reinterpret_cast<const int*>(d)[i];
+  __syncthreads();
+  return *reinterpret_cast<const BDesc*>(s);
+}
+
 // ------------------------------------------------------ spectral passes
 // XMODE: 0 plain x-forward, 1 tangent x-forward.  YINV: y direction.
 // DOT for the x-inverse: 0 none, 1 with dotw, 2 self.
 // cdp, ca, cn (batched like the state, may be NULL): the rank-one part of
 // the symmetric consistent tangent (ConsTan), applied with XMODE 1.
 template <int XMODE>
-__global__ void __launch_bounds__(kXThreads, kXYMinBlocks)
+__global__ void __launch_bounds__(kGT, xy_blocks<R>())
     kb_xfwd(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter,
             const DevScalars* __restrict__ S, const MatTable<R> mt, const R* __restrict__ in,
             const uint8_t* __restrict__ phase, const R* __restrict__ dmg, const R* __restrict__ cdp,
             const R* __restrict__ ca, const R* __restrict__ cn) {
   __shared__ int s_item;
+  __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   for (;;) {
     int v, i, lb;
     if (!fetch(wl, BP_X, counter, &s_item, &v, &i, &lb)) break;
-    const BDesc& d = D[i];
+    const BDesc& d = member_desc(D + i, s_desc);
     const ConsTan<R> ct{cdp ? cdp + d.voff : nullptr, ca ? ca + d.foff : nullptr, cn ? cn + d.foff : nullptr};
     xfwd_body<R, XMODE>(in + d.foff, phase + d.voff, dmg + d.voff, mt, d.spec, d.g, d.qx, d.px, d.tw[0],
                         lb, ct);
@@ -141,56 +152,53 @@ __global__ void __launch_bounds__(kXThreads, kXYMinBlocks)
 }
 
 template <bool YINV>
-__global__ void __launch_bounds__(kYThreads, kXYMinBlocks)
+__global__ void __launch_bounds__(kGT, xy_blocks<R>())
     kb_ycols(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter) {
   __shared__ int s_item;
+  __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   for (;;) {
     int v, i, lb;
     if (!fetch(wl, BP_Y, counter, &s_item, &v, &i, &lb)) break;
-    const BDesc& d = D[i];
-    const int b = lb;
-    const int nbx = (d.g.nxh + d.ty - 1) / d.ty;
-    const int bx = b % nbx, rest = b / nbx;
-    ycols_body<R, YINV>(d.spec, d.g, d.ty, d.py, d.tw[1], bx, rest % d.g.nz, rest / d.g.nz);
+    const BDesc& d = member_desc(D + i, s_desc);
+    ycols_body<R, YINV>(d.spec, d.g, d.lty, d.py, d.tw[1], lb);
   }
 }
 
-__global__ void __launch_bounds__(kZThreads)
+__global__ void __launch_bounds__(kGZ, z_blocks<R>())
     kb_zproj(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter) {
   __shared__ int s_item;
+  __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   for (;;) {
     int v, i, lb;
     if (!fetch(wl, BP_Z, counter, &s_item, &v, &i, &lb)) break;
-    const BDesc& d = D[i];
-    const int b = lb;
-    const int nbx = (d.g.nxh + d.tz - 1) / d.tz;
-    zproj_body<R>(d.spec, d.g, d.tz, d.pz, d.tw[2], d.gd[0], d.ga[0], d.gd[1], d.ga[1], d.gd[2], d.ga[2],
-                  d.free_mask, b % nbx, b / nbx);
+    const BDesc& d = member_desc(D + i, s_desc);
+    zproj_body<R>(d.spec, d.g, d.ltz, d.pz, d.tw[2], d.sy, d.free_mask, lb);
   }
 }
 
-__global__ void __launch_bounds__(kYThreads, kXYMinBlocks)
+__global__ void __launch_bounds__(kGT, xy_blocks<R>())
     kb_yproj2d(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter) {
   __shared__ int s_item;
+  __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   for (;;) {
     int v, i, lb;
     if (!fetch(wl, BP_2D, counter, &s_item, &v, &i, &lb)) break;
-    const BDesc& d = D[i];
-    yproj2d_body<R>(d.spec, d.g, d.tz, d.py, d.tw[1], d.gd[0], d.ga[0], d.gd[1], d.ga[1], d.free_mask,
-                    lb);
+    const BDesc& d = member_desc(D + i, s_desc);
+    yproj2d_body<R>(d.spec, d.g, d.ltz, d.py, d.tw[1], d.sy, d.free_mask, lb);
   }
 }
 
 template <int DOT>
-__global__ void __launch_bounds__(kXThreads, kXYMinBlocks)
+__global__ void __launch_bounds__(kGT, xy_blocks<R>())
     kb_xinv(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter,
             const DevScalars* __restrict__ S, R* __restrict__ out, const R* __restrict__ dotw,
             double* __restrict__ partials) {
   __shared__ int s_item;
+  __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   for (;;) {
     int v, i, lb;
     if (!fetch(wl, BP_X, counter, &s_item, &v, &i, &lb)) break;
-    const BDesc& d = D[i];
+    const BDesc& d = member_desc(D + i, s_desc);
     const R scale = (R)(1.0 / (double)d.g.nvox);
     xinv_body<R, DOT != 0>(d.spec, out + d.foff, DOT == 1 ? dotw + d.foff : nullptr,
                            DOT ? partials + v : nullptr, d.g, d.qx, d.px, d.tw[0], scale, DOT == 2, lb);
@@ -565,40 +573,40 @@ cudaError_t batch_apply(rve_batch_ctx* c, const R* in, R* out, bool tangent, con
     // history change), also inside the captured CG graphs
     const bool cons = c->cdp != nullptr;
     if (tangent)
-      kb_xfwd<1><<<grid_for(tot, kXYMinBlocks), kXThreads, c->smem[BP_X], c->st>>>(
+      kb_xfwd<1><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(
           c->dD, c->wl, next_counter(c), c->S, c->mt, in, c->phase, c->D, cons ? c->cdp : nullptr,
           cons ? c->ca : nullptr, cons ? c->cn : nullptr);
     else
-      kb_xfwd<0><<<grid_for(tot, kXYMinBlocks), kXThreads, c->smem[BP_X], c->st>>>(
+      kb_xfwd<0><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(
           c->dD, c->wl, next_counter(c), c->S, c->mt, in, c->phase, c->D, nullptr, nullptr, nullptr);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (c->any3d) {
-    kb_ycols<false><<<grid_for(c->total[BP_Y], kXYMinBlocks), kYThreads, c->smem[BP_Y], c->st>>>(
+    kb_ycols<false><<<grid_for(c->total[BP_Y], kXYPerSM), kGT, c->smem[BP_Y], c->st>>>(
         c->dD, c->wl, next_counter(c));
-    kb_zproj<<<grid_for(c->total[BP_Z], 2), kZThreads, c->smem[BP_Z], c->st>>>(c->dD, c->wl, next_counter(c));
-    kb_ycols<true><<<grid_for(c->total[BP_Y], kXYMinBlocks), kYThreads, c->smem[BP_Y], c->st>>>(
+    kb_zproj<<<grid_for(c->total[BP_Z], z_blocks<R>()), kGZ, c->smem[BP_Z], c->st>>>(c->dD, c->wl, next_counter(c));
+    kb_ycols<true><<<grid_for(c->total[BP_Y], kXYPerSM), kGT, c->smem[BP_Y], c->st>>>(
         c->dD, c->wl, next_counter(c));
     c->launches += 3;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (c->any2d) {
-    kb_yproj2d<<<grid_for(c->total[BP_2D], kXYMinBlocks), kYThreads, c->smem[BP_2D], c->st>>>(
+    kb_yproj2d<<<grid_for(c->total[BP_2D], kXYPerSM), kGT, c->smem[BP_2D], c->st>>>(
         c->dD, c->wl, next_counter(c));
     ++c->launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const int tot = c->total[BP_X];
   if (!dotw) {
-    kb_xinv<0><<<grid_for(tot, kXYMinBlocks), kXThreads, c->smem[BP_X], c->st>>>(c->dD, c->wl,
+    kb_xinv<0><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl,
                                                                       next_counter(c), c->S, out, nullptr,
                                                                       nullptr);
   } else if (dotw == out) {
-    kb_xinv<2><<<grid_for(tot, kXYMinBlocks), kXThreads, c->smem[BP_X], c->st>>>(c->dD, c->wl,
+    kb_xinv<2><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl,
                                                                       next_counter(c), c->S, out, nullptr,
                                                                       c->part);
   } else {
-    kb_xinv<1><<<grid_for(tot, kXYMinBlocks), kXThreads, c->smem[BP_X], c->st>>>(c->dD, c->wl,
+    kb_xinv<1><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl,
                                                                       next_counter(c), c->S, out, dotw,
                                                                       c->part);
   }
@@ -964,35 +972,32 @@ rve_status batch_init(rve_batch_ctx* c, const int* dims, const int* ndims, const
     d.pz = w.pz;
     for (int a = 0; a < 3; ++a) {
       d.tw[a] = w.tw[a];
-      d.gd[a] = w.gdiff[a];
-      d.ga[a] = w.gavg[a];
+      d.sy.d[a] = w.gdiff[a];
+      d.sy.h[a] = w.gavg[a];
     }
     d.spec = w.spec;
     d.qx = w.qx;
-    d.ty = w.ty;
-    d.tz = w.tz;
+    d.lty = w.lty;
+    d.ltz = w.ltz;
     d.free_mask = 0;
     d.foff = c->nfield;
     d.voff = c->nvox;
     c->nfield += (long long)g.ncomp * g.nvox;
     c->nvox += g.nvox;
+    const GenericTiles<R> gt(g, d.qx, d.lty, d.ltz, d.px, d.py, d.pz);
     const int nb[BP_N] = {
-        (int)((g.nrows + w.qx - 1) / w.qx),
-        g.ndim == 3 ? ((g.nxh + w.ty - 1) / w.ty) * g.nz * g.ncomp : 0,
-        g.ndim == 3 ? ((g.nxh + w.tz - 1) / w.tz) * g.ny : 0,
-        g.ndim == 2 ? (g.nxh + w.tz - 1) / w.tz : 0,
+        gt.xblocks,
+        gt.yblocks,
+        g.ndim == 3 ? gt.zblocks : 0,
+        g.ndim == 2 ? gt.zblocks : 0,
         (int)(((long long)g.ncomp * g.nvox + kVecChunk - 1) / kVecChunk),
         (int)((g.nvox + kVoxChunk - 1) / kVoxChunk),
     };
     for (int p = 0; p < BP_N; ++p) c->hstart[p][i + 1] = c->hstart[p][i] + nb[p];
-    const size_t xs = (size_t)((g.ncomp * w.qx) / 2) * g.nx * sizeof(C);
-    c->smem[BP_X] = std::max(c->smem[BP_X], xs);
-    if (g.ndim == 3) {
-      c->smem[BP_Y] = std::max(c->smem[BP_Y], (size_t)w.ty * g.ny * sizeof(C));
-      c->smem[BP_Z] = std::max(c->smem[BP_Z], (size_t)6 * w.tz * g.nz * sizeof(C));
-    } else {
-      c->smem[BP_2D] = std::max(c->smem[BP_2D], (size_t)3 * w.tz * g.ny * sizeof(C));
-    }
+    c->smem[BP_X] = std::max(c->smem[BP_X], gt.xsmem);
+    c->smem[BP_Y] = std::max(c->smem[BP_Y], gt.ysmem);
+    size_t& zs = c->smem[g.ndim == 3 ? BP_Z : BP_2D];
+    zs = std::max(zs, gt.zsmem);
   }
   std::vector<int> nbh((size_t)BP_N * n);
   for (int p = 0; p < BP_N; ++p) {
@@ -1061,11 +1066,12 @@ rve_status batch_init(rve_batch_ctx* c, const int* dims, const int* ndims, const
 // sx / sy / sz (the tiles of spectral_setup are the largest the per-thread
 // element budgets allow, so only smaller ones are candidates), and the
 // radix order of every axis plan natural or reversed (any order is a valid
-// Stockham factorisation).  Work-item counts, dynamic shared memory, the
+// factorisation).  Work-item counts, dynamic shared memory, the
 // partial-sum buffer and the device descriptors follow; captured graphs are
 // dropped so that they are recaptured with the new schedule.
 void reverse_plan(AxisPlan& p) {
-  for (int a = 0, b = p.nstages - 1; a < b; ++a, --b) std::swap(p.radix[a], p.radix[b]);
+  for (int a = 0, b = p.ns - 1; a < b; ++a, --b) std::swap(p.r[a], p.r[b]);
+  finish_plan(p);
 }
 
 rve_status apply_schedule(rve_batch_ctx* c, const int sched[4]) {
@@ -1079,8 +1085,9 @@ rve_status apply_schedule(rve_batch_ctx* c, const int sched[4]) {
     int qx = std::max(1, w.qx / sched[0]);
     if (g.ncomp & 1) qx = std::max(2, qx & ~1);
     d.qx = qx;
-    d.ty = std::max(1, w.ty / sched[1]);
-    d.tz = std::max(1, w.tz / sched[2]);
+    auto less = [](int l, int div) { return std::max(0, l - (div == 4 ? 2 : div == 2 ? 1 : 0)); };
+    d.lty = less(w.lty, sched[1]);
+    d.ltz = less(w.ltz, sched[2]);
     d.px = w.px;
     d.py = w.py;
     d.pz = w.pz;
@@ -1089,20 +1096,13 @@ rve_status apply_schedule(rve_batch_ctx* c, const int sched[4]) {
       reverse_plan(d.py);
       reverse_plan(d.pz);
     }
-    const int nb[4] = {
-        (int)((g.nrows + d.qx - 1) / d.qx),
-        g.ndim == 3 ? ((g.nxh + d.ty - 1) / d.ty) * g.nz * g.ncomp : 0,
-        g.ndim == 3 ? ((g.nxh + d.tz - 1) / d.tz) * g.ny : 0,
-        g.ndim == 2 ? (g.nxh + d.tz - 1) / d.tz : 0,
-    };
+    const GenericTiles<R> gt(g, d.qx, d.lty, d.ltz, d.px, d.py, d.pz);
+    const int nb[4] = {gt.xblocks, gt.yblocks, g.ndim == 3 ? gt.zblocks : 0, g.ndim == 2 ? gt.zblocks : 0};
     for (int k = 0; k < 4; ++k) c->hstart[passes[k]][i + 1] = c->hstart[passes[k]][i] + nb[k];
-    c->smem[BP_X] = std::max(c->smem[BP_X], (size_t)((g.ncomp * d.qx) / 2) * g.nx * sizeof(C));
-    if (g.ndim == 3) {
-      c->smem[BP_Y] = std::max(c->smem[BP_Y], (size_t)d.ty * g.ny * sizeof(C));
-      c->smem[BP_Z] = std::max(c->smem[BP_Z], (size_t)6 * d.tz * g.nz * sizeof(C));
-    } else {
-      c->smem[BP_2D] = std::max(c->smem[BP_2D], (size_t)3 * d.tz * g.ny * sizeof(C));
-    }
+    c->smem[BP_X] = std::max(c->smem[BP_X], gt.xsmem);
+    c->smem[BP_Y] = std::max(c->smem[BP_Y], gt.ysmem);
+    size_t& zs = c->smem[g.ndim == 3 ? BP_Z : BP_2D];
+    zs = std::max(zs, gt.zsmem);
   }
   std::vector<int> nbh((size_t)BP_N * n);
   for (int p = 0; p < BP_N; ++p) {

@@ -1,5 +1,5 @@
-// Shared device-side definitions: complex helpers, the shared-memory
-// mixed-radix Stockham FFT engine, material tables and block reductions.
+// Shared device-side definitions: complex helpers, radix butterflies,
+// material tables and block reductions.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -29,22 +29,7 @@ template <bool INV, typename C> __device__ __forceinline__ C rot90(C a) {
   return INV ? C{-a.y, a.x} : C{a.y, -a.x};
 }
 
-// ------------------------------------------------------------- FFT plans
-constexpr int kMaxStages = 12;
 constexpr int kMaxPhases = 16;
-
-struct AxisPlan {
-  int n;
-  int nstages;
-  int radix[kMaxStages];
-};
-
-// Line addressing inside a shared-memory tile: line l starts at
-// (l / lpg) * gs + (l % lpg) * ls and its elements are es apart.
-struct LineMap {
-  int lpg, gs, ls, es;
-  __device__ __forceinline__ int base(int l) const { return (l / lpg) * gs + (l % lpg) * ls; }
-};
 
 // ------------------------------------------------------ radix butterflies
 // Small DFTs with the constants of the R-th roots of unity written out.
@@ -127,81 +112,6 @@ template <bool INV, typename C> struct Dft<5, INV, C> {
     a[3] = csub(m2, w2);
   }
 };
-
-// ---------------------------------------------------- Stockham FFT engine
-// One radix-R stage of the self-sorting (Stockham) FFT over `nlines`
-// lines of length n held in shared memory, in place: every thread first
-// loads and transforms its butterflies into registers, the block
-// synchronises, then every thread stores.  Stage with current span Ns:
-// butterfly j of a line reads elements j + r*n/R, multiplies by the
-// twiddle w_n^{r*(j mod Ns)*n/(Ns*R)}, applies the R-point DFT and writes
-// element (j/Ns)*Ns*R + (j mod Ns) + r*Ns.  `LINE_FAST` maps consecutive
-// threads to consecutive lines (for tiles whose lines are interleaved in
-// shared memory) instead of consecutive butterflies of one line.
-template <int R, int EPT, bool INV, bool LINE_FAST, typename C>
-__device__ __forceinline__ void stockham_stage(C* buf, int n, int Ns, int nlines, const LineMap lm,
-                                               const C* __restrict__ tw) {
-  constexpr int MAXB = (EPT + R - 1) / R;
-  const int nbl = n / R;
-  const int total = nlines * nbl;
-  const int tstep = n / (Ns * R);
-  C v[MAXB][R];
-#pragma unroll
-  for (int i = 0; i < MAXB; ++i) {
-    const int b = threadIdx.x + i * blockDim.x;
-    if (b < total) {
-      int l, j;
-      if (LINE_FAST) { j = b / nlines; l = b - j * nlines; }
-      else { l = b / nbl; j = b - l * nbl; }
-      const int k = j % Ns;
-      const int base = lm.base(l);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        C x = buf[base + (j + r * nbl) * lm.es];
-        if (r > 0 && k > 0) {
-          C w = __ldg(&tw[r * k * tstep]);
-          x = INV ? cmulc(x, w) : cmul(x, w);
-        }
-        v[i][r] = x;
-      }
-      Dft<R, INV, C>::run(v[i]);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < MAXB; ++i) {
-    const int b = threadIdx.x + i * blockDim.x;
-    if (b < total) {
-      int l, j;
-      if (LINE_FAST) { j = b / nlines; l = b - j * nlines; }
-      else { l = b / nbl; j = b - l * nbl; }
-      const int k = j % Ns;
-      const int base = lm.base(l);
-      const int d0 = (j / Ns) * Ns * R + k;
-#pragma unroll
-      for (int r = 0; r < R; ++r) buf[base + (d0 + r * Ns) * lm.es] = v[i][r];
-    }
-  }
-  __syncthreads();
-}
-
-// Full transform of every line (forward: sum x_j e^{-2 pi i jk/n}; inverse:
-// conjugate kernel, unnormalised).  Caller synchronises before the call.
-template <int EPT, bool INV, bool LINE_FAST, typename C>
-__device__ void fft_lines(C* buf, const AxisPlan& p, int nlines, const LineMap lm, const C* __restrict__ tw) {
-  int Ns = 1;
-  for (int s = 0; s < p.nstages; ++s) {
-    const int R = p.radix[s];
-    switch (R) {
-      case 8: stockham_stage<8, EPT, INV, LINE_FAST>(buf, p.n, Ns, nlines, lm, tw); break;
-      case 4: stockham_stage<4, EPT, INV, LINE_FAST>(buf, p.n, Ns, nlines, lm, tw); break;
-      case 2: stockham_stage<2, EPT, INV, LINE_FAST>(buf, p.n, Ns, nlines, lm, tw); break;
-      case 3: stockham_stage<3, EPT, INV, LINE_FAST>(buf, p.n, Ns, nlines, lm, tw); break;
-      default: stockham_stage<5, EPT, INV, LINE_FAST>(buf, p.n, Ns, nlines, lm, tw); break;
-    }
-    Ns *= R;
-  }
-}
 
 // ------------------------------------------------------- material tables
 template <typename R> struct MatTable {

@@ -37,7 +37,9 @@ constexpr int fft_radix(int n, int s) {
 }
 constexpr int fft_span(int n, int s) { return s == 0 ? 1 : fft_span(n, s - 1) * fft_radix(n, s - 1); }
 
-// One stage (see stockham_stage in common.cuh for the index scheme).
+// One stage: with span NS done, butterfly j of a line reads elements j + r N/R,
+// multiplies by the twiddle w_N^{r (j mod NS) N/(NS R)}, applies the R-point DFT
+// and writes elements (j/NS) NS R + (j mod NS) + r NS.
 template <int N, int NL, int NT, bool INV, int S, typename C>
 __device__ __forceinline__ void fft_stage_ct(C* buf, const C* __restrict__ tw) {
   constexpr int R = fft_radix(N, S);

@@ -43,23 +43,76 @@ cudaError_t reduce_partials(const double* part, int nblocks, int ns, double* out
 }
 
 // ================================================================ host side
-static void make_plan(int n, AxisPlan& p) {
+void finish_plan(AxisPlan& p) {
+  int span = 1;
+  for (int s = 0; s < p.ns; ++s) {
+    p.span[s] = span;
+    span *= p.r[s];
+    p.m[s] = p.n / span;
+    p.dr[s] = FastDiv::by(p.r[s]);
+    p.dm[s] = FastDiv::by(p.m[s]);
+  }
+  for (int s = 0; s < p.ns; ++s) {
+    p.nw[s] = std::max(1, p.m[0] / p.r[s]);
+    p.dw[s] = FastDiv::by(p.nw[s]);
+  }
+  p.m0p = p.m[0] | 1;
+  p.lp = p.r[0] * p.m0p;
+  p.dn = FastDiv::by(p.n);
+  p.dh = FastDiv::by(p.n / 2 + 1);
+}
+
+// The radix sequence of the compiled passes (8s, 4s, 2, 3s, 5s), successive
+// factors below 8 joined in pairs so that the fewest stages result.
+static void make_plan(int n, AxisPlan& p, bool keep) {
+  p = AxisPlan{};
   p.n = n;
-  p.nstages = 0;
-  int m = n, twos = 0;
+  p.keep_order = keep ? 1 : 0;
+  int f[16], nf = 0, m = n, twos = 0;
   while (m % 2 == 0) { m /= 2; ++twos; }
-  // powers of two: radix 8 as far as possible, then 4 / 4x4 / 2
   int n8 = twos / 3, rem = twos % 3;
   int n4 = 0, n2 = 0;
   if (rem == 2) n4 = 1;
   else if (rem == 1) {
     if (n8 > 0) { --n8; n4 = 2; } else n2 = 1;
   }
-  for (int i = 0; i < n8; ++i) p.radix[p.nstages++] = 8;
-  for (int i = 0; i < n4; ++i) p.radix[p.nstages++] = 4;
-  for (int i = 0; i < n2; ++i) p.radix[p.nstages++] = 2;
-  while (m % 3 == 0) { m /= 3; p.radix[p.nstages++] = 3; }
-  while (m % 5 == 0) { m /= 5; p.radix[p.nstages++] = 5; }
+  for (int i = 0; i < n8; ++i) f[nf++] = 8;
+  for (int i = 0; i < n4; ++i) f[nf++] = 4;
+  for (int i = 0; i < n2; ++i) f[nf++] = 2;
+  while (m % 3 == 0) { m /= 3; f[nf++] = 3; }
+  while (m % 5 == 0) { m /= 5; f[nf++] = 5; }
+  auto pairs = [&](int i) { return i >= 0 && i + 1 < nf && f[i] < 8 && f[i] * f[i + 1] <= 20; };
+  // from the back, and from the front: keep the shorter, then the one with
+  // the smaller largest radix
+  int best[16], nb = 99, mx = 99;
+  for (int side = 0; side < 2; ++side) {
+    int r[16], k = 0;
+    if (side == 0) {
+      for (int i = 0; i < nf; ++i) {
+        if (pairs(i)) { r[k++] = f[i] * f[i + 1]; ++i; }
+        else r[k++] = f[i];
+      }
+    } else {
+      for (int i = nf - 1; i >= 0; --i) {
+        if (pairs(i - 1)) { r[k++] = f[i] * f[i - 1]; --i; }
+        else r[k++] = f[i];
+      }
+      std::reverse(r, r + k);
+    }
+    const int rm = k ? *std::max_element(r, r + k) : 1;
+    if (k < nb || (k == nb && rm < mx)) {
+      nb = k;
+      mx = rm;
+      std::copy(r, r + k, best);
+    }
+  }
+  p.ns = nb;
+  std::copy(best, best + nb, p.r);
+  if (n == 1) {  // an absent axis
+    p.ns = 1;
+    p.r[0] = 1;
+  }
+  finish_plan(p);
 }
 
 template <typename R>
@@ -71,7 +124,10 @@ static cudaError_t upload_tables(int n, Cx<R>** tw, Cx<R>** gdiff, Cx<R>** gavg)
     const long double c = cosl(th), s = sinl(th);
     t[k] = Cx<R>{(R)c, (R)(-s)};
     d[k] = (k == 0) ? Cx<R>{0, 0} : Cx<R>{(R)(c - 1.0L), (R)s};
-    a[k] = (2 * k == n) ? Cx<R>{0, 0} : Cx<R>{(R)((1.0L + c) * 0.5L), (R)(s * 0.5L)};
+    if (std::is_same<R, double>::value)
+      a[k] = Cx<R>{k == 0 ? (R)0 : (R)sinl(0.5L * th), 2 * k == n ? (R)0 : (R)cosl(0.5L * th)};
+    else
+      a[k] = (2 * k == n) ? Cx<R>{0, 0} : Cx<R>{(R)((1.0L + c) * 0.5L), (R)(s * 0.5L)};
   }
   cudaError_t e;
   if ((e = cudaMalloc(tw, n * sizeof(Cx<R>))) != cudaSuccess) return e;
@@ -82,19 +138,77 @@ static cudaError_t upload_tables(int n, Cx<R>** tw, Cx<R>** gdiff, Cx<R>** gavg)
   return cudaMemcpy(*gavg, a.data(), n * sizeof(Cx<R>), cudaMemcpyHostToDevice);
 }
 
-static int pow2_floor(int v) {
-  int p = 1;
-  while (p * 2 <= v) p *= 2;
-  return p;
+template <typename R>
+GenericTiles<R>::GenericTiles(const GridDesc& g, int qx, int lty, int ltz, const AxisPlan& px, const AxisPlan& py,
+                              const AxisPlan& pz) {
+  using C = Cx<R>;
+  xblocks = (int)((g.nrows + qx - 1) / qx);
+  xsmem = (size_t)((g.ncomp * qx) / 2) * px.lp * sizeof(C);
+  if (g.ndim == 3) {
+    yblocks = ColTiles(g.ncomp * g.nz, g.nxh, 1 << lty).count();
+    ysmem = (size_t)(py.lp << lty) * sizeof(C);
+    zblocks = ColTiles(g.ny, g.nxh, 1 << ltz).count();
+    zsmem = (size_t)g.ncomp * (pz.lp << ltz) * sizeof(C);
+  } else {
+    yblocks = 0;
+    ysmem = 0;
+    zblocks = ColTiles(1, g.nxh, 1 << ltz).count();
+    zsmem = (size_t)g.ncomp * (py.lp << ltz) * sizeof(C);
+  }
+}
+template struct GenericTiles<float>;
+template struct GenericTiles<double>;
+
+// Plans and tiles.  A tile is as large as keeps its threads busy (about one
+// butterfly each, 128-byte column segments) and as small as leaves every SM
+// work: with one tile size for all grids, each pass of a 32^2 cell ran on ONE
+// SM (FP64 product 129 -> 35 us with 16-17 blocks per pass).  Columns do not
+// go below the 32 bytes of a memory sector while a tile fits a block.
+template <typename R>
+cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w) {
+  using C = Cx<R>;
+  // FP32 cells of one element per voxel keep their roundings (zproj_body)
+  const bool keep = std::is_same<R, float>::value && g.nq == 1;
+  make_plan(g.nx, w.px, keep);
+  make_plan(g.ny, w.py, keep);
+  make_plan(g.ndim == 3 ? g.nz : 1, w.pz, keep);
+  w.px.dc = FastDiv::by(g.ncomp);
+  const int wave = 2 * 152;              // blocks that give every SM two
+  const int q1 = (g.ncomp & 1) ? 2 : 1;  // rows come in pairs where ncomp is odd
+  // x: about 2048 elements (16 KB in FP32) per block
+  long long q = std::max<long long>(q1, 2 * 2048 / ((long long)g.ncomp * g.nx));
+  q = std::min<long long>(q, std::max<long long>(q1, g.nrows / wave));
+  w.qx = (int)((g.ncomp & 1) ? std::max<long long>(2, q & ~1LL) : q);
+  const int lseg = sizeof(C) == 8 ? 4 : 3, lsec = lseg - 2;  // columns of 128 and of 32 bytes (log2)
+  // hold: elements per line group that one block's threads can reorder
+  auto columns = [&](const AxisPlan& p, int groups, int planes, int elems, int hold) {
+    int l = 7;  // short lines: up to 128 columns, so that a tile keeps its threads busy
+    while (l > lseg && ((long long)groups * p.n << l) > 2048) --l;
+    while (l > 0 && (((size_t)groups * (p.lp << l) * sizeof(C) > (size_t)kSmemCap) || (keep && (p.n << l) > hold))) --l;
+    while (l > lsec && ((long long)groups * p.n << l) > elems) --l;
+    while (l > 0 && ColTiles(planes, g.nxh, 1 << l).count() < wave) --l;
+    return l;
+  };
+  w.lty = g.ndim == 3 ? columns(w.py, 1, g.ncomp * g.nz, 4096, 1 << 30) : 0;
+  if (g.ndim == 3) w.ltz = columns(w.pz, g.ncomp, g.ny, sizeof(C) == 8 ? 6144 : 3072, kHold * kGZ);
+  else w.ltz = columns(w.py, g.ncomp, 1, 3072, kHold2 * kGT);
+  // opt in to large dynamic shared memory
+  cudaFuncSetAttribute(k_xfwd<R, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+  cudaFuncSetAttribute(k_xfwd<R, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+  cudaFuncSetAttribute(k_ycols<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+  cudaFuncSetAttribute(k_ycols<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+  cudaFuncSetAttribute(k_zproj<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+  cudaFuncSetAttribute(k_yproj2d<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+  cudaFuncSetAttribute(k_xinv<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+  cudaFuncSetAttribute(k_xinv<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+  return cudaGetLastError();
 }
 
 template <typename R>
 cudaError_t spectral_setup(const GridDesc& g, SpecWork<R>& w) {
   using C = Cx<R>;
-  make_plan(g.nx, w.px);
-  make_plan(g.ny, w.py);
-  make_plan(g.ndim == 3 ? g.nz : 1, w.pz);
-  cudaError_t e;
+  cudaError_t e = spectral_plan<R>(g, w);
+  if (e != cudaSuccess) return e;
   const int ns[3] = {g.nx, g.ny, g.nz};
   for (int a = 0; a < g.ndim; ++a)
     if ((e = upload_tables<R>(ns[a], &w.tw[a], &w.gdiff[a], &w.gavg[a])) != cudaSuccess) return e;
@@ -111,68 +225,10 @@ cudaError_t spectral_setup(const GridDesc& g, SpecWork<R>& w) {
     if ((e = cudaMalloc(&w.twq, m * sizeof(C))) != cudaSuccess) return e;
     if ((e = cudaMemcpy(w.twq, t.data(), m * sizeof(C), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
   }
-  // x passes: npair * nx <= kXThreads * kXEpt complex per block
-  const int ex = kXThreads * kXEpt;
-  int q = (2 * ex) / (g.ncomp * g.nx);
-  if (g.ncomp & 1) q &= ~1;
-  q = std::max(q, (g.ncomp & 1) ? 2 : 1);
-  w.qx = (int)std::min<long long>(q, g.nrows + (g.nrows & 1));
-  // y columns
-  const int ey = kYThreads * kYEpt;
-  w.ty = std::max(1, std::min(pow2_floor(std::max(1, ey / g.ny)), 64));
-  // z + projection (3D) or y + projection (2D)
-  if (g.ndim == 3) {
-    const int ez = std::min(kZThreads * kZEpt, (int)(kSmemCap / sizeof(C)));
-    w.tz = std::max(1, std::min(pow2_floor(std::max(1, ez / (g.ncomp * g.nz))), 16));
-  } else {
-    const int e2 = std::min(kYThreads * kYEpt, (int)(kSmemCap / sizeof(C)));
-    w.tz = std::max(1, std::min(pow2_floor(std::max(1, e2 / (g.ncomp * g.ny))), 64));
-  }
-  // up to three partial sums per x block (the fused CG x-inverse), and the
-  // compile-time x passes may take a single row per block (Nx = 512)
+  // up to three partial sums per x block (the fused CG x-inverse), and an x
+  // block may hold a single row
   w.max_partials = (int)std::max<long long>(3 * g.nrows + 8, 4096 * 8);
-  if ((e = cudaMalloc(&w.partials, (size_t)w.max_partials * sizeof(double))) != cudaSuccess) return e;
-  // opt in to large dynamic shared memory
-  cudaFuncSetAttribute(k_xfwd<R, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_xfwd<R, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_ycols<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_ycols<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_zproj<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_yproj2d<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_xinv<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_xinv<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  return cudaGetLastError();
-}
-
-// Plans and tile sizes for a caller that brings its own tables and spectrum
-// storage (no device allocation): the same choices as spectral_setup.
-template <typename R>
-cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w) {
-  using C = Cx<R>;
-  make_plan(g.nx, w.px);
-  make_plan(g.ny, w.py);
-  make_plan(g.ndim == 3 ? g.nz : 1, w.pz);
-  const int ex = kXThreads * kXEpt;
-  int q = (2 * ex) / (g.ncomp * g.nx);
-  if (g.ncomp & 1) q &= ~1;
-  q = std::max(q, (g.ncomp & 1) ? 2 : 1);
-  w.qx = (int)std::min<long long>(q, g.nrows + (g.nrows & 1));
-  const int ey = kYThreads * kYEpt;
-  w.ty = std::max(1, std::min(pow2_floor(std::max(1, ey / g.ny)), 64));
-  if (g.ndim == 3) {
-    const int ez = std::min(kZThreads * kZEpt, (int)(kSmemCap / sizeof(C)));
-    w.tz = std::max(1, std::min(pow2_floor(std::max(1, ez / (g.ncomp * g.nz))), 16));
-  } else {
-    const int e2 = std::min(kYThreads * kYEpt, (int)(kSmemCap / sizeof(C)));
-    w.tz = std::max(1, std::min(pow2_floor(std::max(1, e2 / (g.ncomp * g.ny))), 64));
-  }
-  cudaFuncSetAttribute(k_xfwd<R, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_ycols<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_ycols<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_zproj<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_yproj2d<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  cudaFuncSetAttribute(k_xinv<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-  return cudaGetLastError();
+  return cudaMalloc(&w.partials, (size_t)w.max_partials * sizeof(double));
 }
 
 template <typename R>
@@ -200,11 +256,9 @@ static cudaError_t spectral_middle(const GridDesc& g, SpecWork<R>& w, cudaStream
   constexpr bool F32 = std::is_same<R, float>::value;
   long long nl = 0;
   cudaError_t e;
+  const GenericTiles<R> gt(g, w.qx, w.lty, w.ltz, w.px, w.py, w.pz);
+  const AxisSyms<R> sy{{w.gdiff[0], w.gdiff[1], w.gdiff[2]}, {w.gavg[0], w.gavg[1], w.gavg[2]}};
   if (g.ndim == 3) {
-    const dim3 yg((g.nxh + w.ty - 1) / w.ty, g.nz, g.ncomp);
-    const size_t ysm = (size_t)w.ty * g.ny * sizeof(C);
-    const dim3 zg((g.nxh + w.tz - 1) / w.tz, g.ny);
-    const size_t zsm = (size_t)g.ncomp * w.tz * g.nz * sizeof(C);
     for (int pass = 0; pass < 3; ++pass) {
       if ((pass == 0 && skip_yfwd) || (pass == 2 && skip_yinv)) continue;  // done by the cluster x+y passes
       e = cudaErrorNotSupported;
@@ -214,11 +268,9 @@ static cudaError_t spectral_middle(const GridDesc& g, SpecWork<R>& w, cudaStream
         if (!w.generic && pass == 1 && fast_size(g.nz)) e = fast_zproj(g, w.spec, w, st);
       }
       if (e == cudaErrorNotSupported) {
-        if (pass == 0) k_ycols<R, false><<<yg, kYThreads, ysm, st>>>(w.spec, g, w.ty, w.py, w.tw[1]);
-        else if (pass == 2) k_ycols<R, true><<<yg, kYThreads, ysm, st>>>(w.spec, g, w.ty, w.py, w.tw[1]);
-        else
-          k_zproj<R><<<zg, kZThreads, zsm, st>>>(w.spec, g, w.tz, w.pz, w.tw[2], w.gdiff[0], w.gavg[0],
-                                                 w.gdiff[1], w.gavg[1], w.gdiff[2], w.gavg[2], w.free_mask);
+        if (pass == 0) k_ycols<R, false><<<gt.yblocks, kGT, gt.ysmem, st>>>(w.spec, g, w.lty, w.py, w.tw[1]);
+        else if (pass == 2) k_ycols<R, true><<<gt.yblocks, kGT, gt.ysmem, st>>>(w.spec, g, w.lty, w.py, w.tw[1]);
+        else k_zproj<R><<<gt.zblocks, kGZ, gt.zsmem, st>>>(w.spec, g, w.ltz, w.pz, w.tw[2], sy, w.free_mask);
         e = cudaGetLastError();
       }
       if (e != cudaSuccess) return e;
@@ -231,10 +283,7 @@ static cudaError_t spectral_middle(const GridDesc& g, SpecWork<R>& w, cudaStream
       if (!w.generic && fast_size(g.ny)) e = fast_yproj2d(g, w.spec, w, st);
     }
     if (e == cudaErrorNotSupported) {
-      const dim3 pg((g.nxh + w.tz - 1) / w.tz);
-      const size_t psm = (size_t)g.ncomp * w.tz * g.ny * sizeof(C);
-      k_yproj2d<R><<<pg, kYThreads, psm, st>>>(w.spec, g, w.tz, w.py, w.tw[1], w.gdiff[0], w.gavg[0], w.gdiff[1],
-                                               w.gavg[1], w.free_mask);
+      k_yproj2d<R><<<gt.zblocks, kGT, gt.zsmem, st>>>(w.spec, g, w.ltz, w.py, w.tw[1], sy, w.free_mask);
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
@@ -259,8 +308,9 @@ cudaError_t spectral_apply(const GridDesc& g, SpecWork<R>& w, const MatTable<R>&
   constexpr bool F32 = std::is_same<R, float>::value;
   long long nl = 0;
   cudaError_t e;
-  const int xblocks = (int)((g.nrows + w.qx - 1) / w.qx);
-  const size_t xsm = (size_t)((g.ncomp * w.qx) / 2) * g.nx * sizeof(C);
+  const GenericTiles<R> gt(g, w.qx, w.lty, w.ltz, w.px, w.py, w.pz);
+  const int xblocks = gt.xblocks;
+  const size_t xsm = gt.xsmem;
   // dot(in, G:B:in) for a compatible input (in = G:in, as every CG direction
   // is) equals dot(in, B:in): the compiled x-forward pass forms it from the
   // tangent it already computes, so the x-inverse need not read `in` again
@@ -294,9 +344,9 @@ cudaError_t spectral_apply(const GridDesc& g, SpecWork<R>& w, const MatTable<R>&
   }
   if (e == cudaErrorNotSupported) {
     if (mode == XIn::Tangent)
-      k_xfwd<R, 1><<<xblocks, kXThreads, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0], w.cons);
+      k_xfwd<R, 1><<<xblocks, kGT, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0], w.cons);
     else
-      k_xfwd<R, 0><<<xblocks, kXThreads, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0],
+      k_xfwd<R, 0><<<xblocks, kGT, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0],
                                                     ConsTan<R>{});
     e = cudaGetLastError();
   }
@@ -322,10 +372,10 @@ cudaError_t spectral_apply(const GridDesc& g, SpecWork<R>& w, const MatTable<R>&
   if (e == cudaErrorNotSupported) {
     nblocks = xblocks;
     if (dot)
-      k_xinv<R, true><<<xblocks, kXThreads, xsm, st>>>(w.spec, out, self ? nullptr : dot_with, w.partials, g, w.qx,
+      k_xinv<R, true><<<xblocks, kGT, xsm, st>>>(w.spec, out, self ? nullptr : dot_with, w.partials, g, w.qx,
                                                        w.px, w.tw[0], scale, self);
     else
-      k_xinv<R, false><<<xblocks, kXThreads, xsm, st>>>(w.spec, out, nullptr, nullptr, g, w.qx, w.px, w.tw[0],
+      k_xinv<R, false><<<xblocks, kGT, xsm, st>>>(w.spec, out, nullptr, nullptr, g, w.qx, w.px, w.tw[0],
                                                         scale, false);
     e = cudaGetLastError();
   }

@@ -2,6 +2,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "fft_inplace.cuh"
 #include "pass_timer.cuh"
 
 namespace rve {
@@ -30,16 +31,15 @@ template <typename R> struct ConsTan {
 
 // Tables and workspace for the spectral passes at precision R.
 template <typename R> struct SpecWork {
-  AxisPlan px, py, pz;
+  AxisPlan px{}, py{}, pz{};
   Cx<R>* tw[3] = {nullptr, nullptr, nullptr};    // e^{-2 pi i t / n_axis}
   Cx<R>* gdiff[3] = {nullptr, nullptr, nullptr}; // e^{i th} - 1 (exact 0 at k=0)
-  Cx<R>* gavg[3] = {nullptr, nullptr, nullptr};  // (1 + e^{i th})/2 (exact 0 at 2k=n)
+  Cx<R>* gavg[3] = {nullptr, nullptr, nullptr};  // FP32: (1 + e^{i th})/2; FP64: (sin, cos)(th/2) (AxisSyms)
   Cx<R>* spec = nullptr;                          // ncomp * nz * ny * nxh
   unsigned free_mask = 0;                         // bit c: Mandel comp c stress-controlled
-  // tiling
-  int qx;   // voxel rows per x-pass block
-  int ty;   // kx columns per y-pass block
-  int tz;   // kx columns per z-pass / 2D y-pass block
+  // tiling of the generic passes
+  int qx;        // voxel rows per x-pass block
+  int lty, ltz;  // log2 of the kx columns per y-pass block, per z-pass / 2D y-pass block
   double* partials = nullptr;  // per-block FP64 partial sums (epilogues)
   int max_partials = 0;
   PassTimer* timer = nullptr;  // optional per-pass event timing
@@ -84,6 +84,16 @@ void spectral_free(SpecWork<R>& w);
 // the tables and the spectrum storage in SpecWork).
 template <typename R>
 cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w);
+// Tile sizes and the blocks / dynamic shared memory they give, for the
+// generic passes with these plans.
+template <typename R> struct GenericTiles {
+  int xblocks, yblocks, zblocks;  // zblocks: the 2D y pass in 2D
+  size_t xsmem, ysmem, zsmem;
+  GenericTiles(const GridDesc& g, int qx, int lty, int ltz, const AxisPlan& px, const AxisPlan& py,
+               const AxisPlan& pz);
+};
+// Stage tables of a plan from its radices.
+void finish_plan(AxisPlan& p);
 
 // FP64 final reduction of per-block partials: out[s] = sum_b part[b*ns + s]
 // (out: ns contiguous device doubles).  Fixed summation order.

@@ -1,23 +1,25 @@
 // Generic (runtime-length) spectral pass bodies and their single-grid
-// kernels.  A body processes one block of one grid; the kernels call it with
+// kernels.  A body processes one tile of one grid; the kernels call it with
 // their block index, batched kernels with an index taken from a work list.
 #pragma once
 
+#include "fft_inplace.cuh"
 #include "hv_passes.cuh"
 #include "project.cuh"
 
 namespace rve {
 
-constexpr int kXThreads = 256, kXEpt = 16;  // x passes
-constexpr int kYThreads = 256, kYEpt = 16;  // y columns, 2D y+projection
-constexpr int kZThreads = 512, kZEpt = 24;  // z + projection
-constexpr int kSmemCap = 100 * 1024;        // dynamic shared memory cap per block
-// The x and y kernels are compiled for six resident blocks per SM (at most
-// 42 registers a thread): their runtime-radix stages otherwise take 200-255
-// registers and leave one block (8 warps) per SM, latency-bound.  The spills
-// this costs are cheaper than the idle SM (2.4x faster generic passes at
-// 256^3 FP32, 1.3x in FP64 at 128^3).
-constexpr int kXYMinBlocks = 6;
+constexpr int kSmemCap = 112 * 1024;  // dynamic shared memory cap per block: two blocks fit an SM
+constexpr int kGT = 128;              // threads of the x, y and 2D passes
+constexpr int kGZ = 256;              // threads of the z pass
+constexpr int kHold = 4, kHold2 = 8;  // frequencies a z-pass / 2D y-pass thread holds while its tile is reordered
+
+// One butterfly per thread in registers (radix <= 20: 40 reals) leaves no
+// reason to cap the registers hard: 24 resident warps of FP32 at 80 registers
+// and 16 of FP64 at 128 (whose passes are bound by the FP64 pipe, 2 lanes per
+// SM and clock, not by latency) are asked for.
+template <typename R> constexpr int xy_blocks() { return sizeof(R) == 4 ? 6 : 4; }
+template <typename R> constexpr int z_blocks() { return sizeof(R) == 4 ? 3 : 2; }
 
 // ------------------------------------------------------------ x forward
 // Q voxel rows per block, all ncomp components of each row.  With the
@@ -35,34 +37,42 @@ __device__ __forceinline__ void xfwd_body(const R* __restrict__ in, const uint8_
   using C = Cx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  const int nx = g.nx, nc = g.ncomp, nd = g.ndim;
+  const int nx = g.nx, nc = g.ncomp, nd = g.ndim, lp = px.lp;
   const long long row0 = (long long)bx * Q;
   const int npair = (nc * Q) >> 1;
   for (int idx = threadIdx.x; idx < Q * nx; idx += blockDim.x) {
-    const int q = idx / nx, x = idx - q * nx;
+    const int q = px.dn.div(idx), x = idx - q * nx;
+    const int at = px.at_natural(x);
     const long long row = row0 + q;
     if (g.nq > 1) {
       // Kuhn simplices: line c * nq + p is Mandel component c of simplex p,
       // whose damage is dmg[p * nvox + vox]; the tangent acts per simplex
-      const int nqp = g.nq, nm = nc / nqp;
+      const int nqp = g.nq, nm = nd == 3 ? 6 : 3;
       const long long vox = row * nx + x;
       for (int p = 0; p < nqp; ++p) {
         R m[6] = {0, 0, 0, 0, 0, 0};
         if (row < g.nrows) {
-          for (int c = 0; c < nm; ++c) m[c] = in[(c * nqp + p) * g.nvox + vox];
+#pragma unroll
+          for (int c = 0; c < 6; ++c)
+            if (c < nm) m[c] = in[(c * nqp + p) * g.nvox + vox];
           if (MODE == 1) {
             const int ph = phase[vox];
             const R keep = (R)1 - dmg[p * g.nvox + vox];
             const R lam = mt.lam[ph] * keep, two_mu = (R)2 * mt.mu[ph] * keep;
             R tr = 0;
-            for (int i = 0; i < nd; ++i) tr += m[i];
-            for (int c = 0; c < nm; ++c) m[c] = two_mu * m[c] + (c < nd ? lam * tr : (R)0);
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+              if (i < nd) tr += m[i];
+#pragma unroll
+            for (int c = 0; c < 6; ++c) m[c] = two_mu * m[c] + (c < nd ? lam * tr : (R)0);
           }
         }
-        for (int c = 0; c < nm; ++c) {
-          const int rho = q * nc + c * nqp + p;
-          R* slot = reinterpret_cast<R*>(&buf[(rho >> 1) * nx + x]) + (rho & 1);
-          *slot = m[c];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          if (c < nm) {
+            const int rho = q * nc + c * nqp + p;
+            reinterpret_cast<R*>(&buf[(rho >> 1) * lp + at])[rho & 1] = m[c];
+          }
         }
       }
       continue;
@@ -70,13 +80,17 @@ __device__ __forceinline__ void xfwd_body(const R* __restrict__ in, const uint8_
     R val[6] = {0, 0, 0, 0, 0, 0};
     if (row < g.nrows) {
       const long long vox = row * nx + x;
-      for (int c = 0; c < nc; ++c) val[c] = in[c * g.nvox + vox];
+#pragma unroll
+      for (int c = 0; c < 6; ++c)
+        if (c < nc) val[c] = in[c * g.nvox + vox];
       if (MODE == 1) {
         const int ph = phase[vox];
         const R keep = (R)1 - dmg[vox];
         const R lam = mt.lam[ph] * keep, two_mu = (R)2 * mt.mu[ph] * keep;
         R tr = 0;
-        for (int i = 0; i < nd; ++i) tr += val[i];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          if (i < nd) tr += val[i];
         const R hdp = ct.dp ? (R)0.5 * ct.dp[vox] : (R)0;
         R nv = 0, av = 0;
         if (hdp != (R)0) {
@@ -85,31 +99,36 @@ __device__ __forceinline__ void xfwd_body(const R* __restrict__ in, const uint8_
             av += ct.a[c * g.nvox + vox] * val[c];
           }
         }
-        for (int c = 0; c < nc; ++c) {
-          val[c] = two_mu * val[c] + (c < nd ? lam * tr : (R)0);
-          if (hdp != (R)0) val[c] -= hdp * (ct.a[c * g.nvox + vox] * nv + ct.n[c * g.nvox + vox] * av);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          if (c < nc) {
+            val[c] = two_mu * val[c] + (c < nd ? lam * tr : (R)0);
+            if (hdp != (R)0) val[c] -= hdp * (ct.a[c * g.nvox + vox] * nv + ct.n[c * g.nvox + vox] * av);
+          }
         }
       }
     }
-    for (int c = 0; c < nc; ++c) {
-      const int rho = q * nc + c;
-      R* slot = reinterpret_cast<R*>(&buf[(rho >> 1) * nx + x]) + (rho & 1);
-      *slot = val[c];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      if (c < nc) {
+        const int rho = q * nc + c;
+        reinterpret_cast<R*>(&buf[(rho >> 1) * lp + at])[rho & 1] = val[c];
+      }
     }
   }
   __syncthreads();
-  fft_lines<kXEpt, false, false>(buf, px, npair, LineMap{1, nx, 0, 1}, tw);
+  tile_dit<false, false, false>(buf, px, TileShape{npair, 1, 0}, tw, NoIo{}, NoIo{});
   const int nxh = g.nxh;
   for (int idx = threadIdx.x; idx < npair * nxh; idx += blockDim.x) {
-    const int p = idx / nxh, k = idx - p * nxh;
-    const C zk = buf[p * nx + k];
-    const C zm = buf[p * nx + (k == 0 ? 0 : nx - k)];
+    const int p = px.dh.div(idx), k = idx - p * nxh;
+    const C zk = buf[p * lp + px.at_freq(k)];
+    const C zm = buf[p * lp + px.at_freq(k == 0 ? 0 : nx - k)];
     const C xa = C{(zk.x + zm.x) * (R)0.5, (zk.y - zm.y) * (R)0.5};
     const C xb = C{(zk.y + zm.y) * (R)0.5, (zm.x - zk.x) * (R)0.5};
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int rho = 2 * p + h;
-      const int q = rho / nc, c = rho - q * nc;
+      const int q = px.dc.div(rho), c = rho - q * nc;
       const long long row = row0 + q;
       if (q < Q && row < g.nrows) spec[(c * g.nrows + row) * nxh + k] = h ? xb : xa;
     }
@@ -117,168 +136,217 @@ __device__ __forceinline__ void xfwd_body(const R* __restrict__ in, const uint8_
 }
 
 template <typename R, int MODE>
-__global__ void __launch_bounds__(kXThreads, kXYMinBlocks)
+__global__ void __launch_bounds__(kGT, xy_blocks<R>())
     k_xfwd(const R* __restrict__ in, const uint8_t* __restrict__ phase, const R* __restrict__ dmg,
-           const MatTable<R> mt, Cx<R>* __restrict__ spec, const GridDesc g, const int Q, const AxisPlan px,
-           const Cx<R>* __restrict__ tw, const ConsTan<R> ct) {
+           const MatTable<R> mt, Cx<R>* __restrict__ spec, const GridDesc g, const int Q,
+           const __grid_constant__ AxisPlan px, const Cx<R>* __restrict__ tw, const ConsTan<R> ct) {
   xfwd_body<R, MODE>(in, phase, dmg, mt, spec, g, Q, px, tw, blockIdx.x, ct);
 }
 
 // ------------------------------------------------------------ y columns
+// One tile of TX kx columns of the planes (component, z), transformed in
+// global memory.
 template <typename R, bool INV>
-__device__ __forceinline__ void ycols_body(Cx<R>* __restrict__ spec, const GridDesc& g, const int TX,
-                                           const AxisPlan& py, const Cx<R>* __restrict__ tw, const int bx,
-                                           const int by, const int bz) {
+__device__ __forceinline__ void ycols_body(Cx<R>* __restrict__ spec, const GridDesc& g, const int ltx,
+                                           const AxisPlan& py, const Cx<R>* __restrict__ tw, const int b) {
   using C = Cx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  const int ny = g.ny, nxh = g.nxh;
-  const int kx0 = bx * TX;
-  const int tv = min(TX, nxh - kx0);
-  const long long plane = ((long long)bz * g.nz + by) * ny;
-  for (int idx = threadIdx.x; idx < ny * TX; idx += blockDim.x) {
-    const int y = idx / TX, t = idx - y * TX;
-    buf[idx] = t < tv ? spec[(plane + y) * nxh + kx0 + t] : C{0, 0};
-  }
-  __syncthreads();
-  fft_lines<kYEpt, INV, true>(buf, py, TX, LineMap{TX, 0, 1, TX}, tw);
-  for (int idx = threadIdx.x; idx < ny * TX; idx += blockDim.x) {
-    const int y = idx / TX, t = idx - y * TX;
-    if (t < tv) spec[(plane + y) * nxh + kx0 + t] = buf[idx];
-  }
+  const int tx = 1 << ltx, nxh = g.nxh;
+  // the threads are a multiple of the columns: a thread keeps one column
+  int plane, kx;
+  const bool ok = ColTiles(g.ncomp * g.nz, nxh, tx).at(b, threadIdx.x & (tx - 1), &plane, &kx);
+  C* col = spec + (long long)plane * g.ny * nxh + kx;
+  auto load = [=](int, int y, int) -> C { return ok ? col[(long long)y * nxh] : C{0, 0}; };
+  auto store = [=](int, int y, int, C v) {
+    if (ok) col[(long long)y * nxh] = v;
+  };
+  tile_dit<INV, true, true>(buf, py, TileShape{1, tx, ltx}, tw, load, store);
 }
 
 template <typename R, bool INV>
-__global__ void __launch_bounds__(kYThreads, kXYMinBlocks)
-    k_ycols(Cx<R>* __restrict__ spec, const GridDesc g, const int TX, const AxisPlan py,
+__global__ void __launch_bounds__(kGT, xy_blocks<R>())
+    k_ycols(Cx<R>* __restrict__ spec, const GridDesc g, const int ltx, const __grid_constant__ AxisPlan py,
             const Cx<R>* __restrict__ tw) {
-  ycols_body<R, INV>(spec, g, TX, py, tw, blockIdx.x, blockIdx.y, blockIdx.z);
+  ycols_body<R, INV>(spec, g, ltx, py, tw, blockIdx.x);
 }
 
 // ------------------------------------------------- z + projection (3D)
+// One tile of kx columns at ky, all components: z transform, projection,
+// inverse z transform.
+//
+// pz.keep_order (FP32 cells of one element per voxel): the inverse runs the
+// forward's radix sequence from natural order, so that every value is formed
+// by the same operations in the same order as in earlier releases of this
+// pass (an FP32 load path follows its roundings).  The tile is reordered
+// through registers with the projection (kHold frequencies per thread).
+// Otherwise the inverse is the transposed flow and nothing is reordered.
 template <typename R>
-__device__ __forceinline__ void zproj_body(Cx<R>* __restrict__ spec, const GridDesc& g, const int TX,
-                                           const AxisPlan& pz, const Cx<R>* __restrict__ tw,
-                                           const Cx<R>* __restrict__ gdx, const Cx<R>* __restrict__ gax,
-                                           const Cx<R>* __restrict__ gdy, const Cx<R>* __restrict__ gay,
-                                           const Cx<R>* __restrict__ gdz, const Cx<R>* __restrict__ gaz,
-                                           const unsigned free_mask, const int bx, const int by) {
+__device__ __forceinline__ void zproj_body(Cx<R>* __restrict__ spec, const GridDesc& g, const int ltx,
+                                           const AxisPlan& pz, const Cx<R>* __restrict__ tw, const AxisSyms<R>& sy,
+                                           const unsigned free_mask, const int b) {
   using C = Cx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  const int nz = g.nz, ny = g.ny, nxh = g.nxh;
+  const int nz = g.nz, ny = g.ny, nxh = g.nxh, tx = 1 << ltx;
   const int ncl = g.ncomp;  // lines per column: 6, or 36 for Kuhn tetrahedra
-  const int kx0 = bx * TX, ky = by;
-  const int tv = min(TX, nxh - kx0);
-  const int plane = nz * TX;
-  for (int idx = threadIdx.x; idx < ncl * plane; idx += blockDim.x) {
-    const int c = idx / plane, rem = idx - c * plane;
-    const int z = rem / TX, t = rem - z * TX;
-    buf[idx] = t < tv ? spec[(((long long)c * nz + z) * ny + ky) * nxh + kx0 + t] : C{0, 0};
-  }
-  __syncthreads();
-  const LineMap lm{TX, plane, 1, TX};
-  fft_lines<kZEpt, false, true>(buf, pz, ncl * TX, lm, tw);
-  const C ay = gay[ky], dy = gdy[ky];
-  for (int pt = threadIdx.x; pt < plane; pt += blockDim.x) {
-    const int z = pt / TX, t = pt - z * TX;
-    const int kx = kx0 + t;
-    if (t >= tv) continue;
-    if (ncl == 36) {
-      const C d[3] = {gdx[kx], dy, gdz[z]};
-      const C e[3] = {C{(R)1 + d[0].x, d[0].y}, C{(R)1 + d[1].x, d[1].y}, C{(R)1 + d[2].x, d[2].y}};
-      project_simplex3<R>(buf + pt, plane, e, d, kx == 0 && ky == 0 && z == 0, free_mask);
-      continue;
+  const int t = threadIdx.x & (tx - 1);
+  int ky, kx;
+  const bool ok = ColTiles(ny, nxh, tx).at(b, t, &ky, &kx);
+  const long long zs = (long long)ny * nxh;
+  C* col = spec + (long long)ky * nxh + kx;
+  auto load = [=](int c, int z, int) -> C { return ok ? col[(c * nz + z) * zs] : C{0, 0}; };
+  auto store = [=](int c, int z, int, C v) {
+    if (ok) col[(c * nz + z) * zs] = v;
+  };
+  const TileShape ts{ncl, tx, ltx};
+  tile_dit<false, true, false>(buf, pz, ts, tw, load, NoIo{});
+  const bool kxy0 = kx == 0 && ky == 0;
+  const int lp = pz.lp << ltx;
+  if (ncl == 36) {
+    if (ok) {
+      for (int i = threadIdx.x >> ltx; i < nz; i += blockDim.x >> ltx) {
+        const int e = pz.dr[0].div(i), q0 = i - e * pz.r[0], z = pz.freq_of(q0, e);
+        const C d[3] = {sy.d[0][kx], sy.d[1][ky], sy.d[2][z]};
+        const C ex[3] = {C{(R)1 + d[0].x, d[0].y}, C{(R)1 + d[1].x, d[1].y}, C{(R)1 + d[2].x, d[2].y}};
+        project_simplex3<R>(buf + ((q0 * pz.m0p + e) << ltx) + t, lp, ex, d, kxy0 && z == 0, free_mask);
+      }
     }
-    C m[6];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) m[c] = buf[c * plane + pt];
-    const C ax = gax[kx], dx = gdx[kx], az = gaz[z], dz = gdz[z];
-    const C d0 = cmul(cmul(dx, ay), az);
-    const C d1 = cmul(cmul(ax, dy), az);
-    const C d2 = cmul(cmul(ax, ay), dz);
-    project3<R>(m, d0, d1, d2, kx == 0 && ky == 0 && z == 0, free_mask);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) buf[c * plane + pt] = m[c];
+    __syncthreads();
+    tile_transposed_inverse(buf, pz, ts, tw, store);
+    return;
   }
-  __syncthreads();
-  fft_lines<kZEpt, true, true>(buf, pz, ncl * TX, lm, tw);
-  for (int idx = threadIdx.x; idx < ncl * plane; idx += blockDim.x) {
-    const int c = idx / plane, rem = idx - c * plane;
-    const int z = rem / TX, t = rem - z * TX;
-    if (t < tv) spec[(((long long)c * nz + z) * ny + ky) * nxh + kx0 + t] = buf[idx];
+  const ColSym3<R> cs = ok ? ColSym3<R>(sy, kx, ky) : ColSym3<R>();
+  if (!pz.keep_order) {
+    if (ok) {
+      for (int i = threadIdx.x >> ltx; i < nz; i += blockDim.x >> ltx) {
+        const int e = pz.dr[0].div(i), q0 = i - e * pz.r[0], z = pz.freq_of(q0, e);
+        C* at = buf + ((q0 * pz.m0p + e) << ltx) + t;
+        C m[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) m[c] = at[c * lp];
+        cs.project(m, sy, z, kxy0 && z == 0, free_mask);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) at[c * lp] = m[c];
+      }
+    }
+    __syncthreads();
+    tile_transposed_inverse(buf, pz, ts, tw, store);
+    return;
+  }
+  if constexpr (sizeof(R) == 4) {
+    C m[kHold][6];
+#pragma unroll
+    for (int h = 0; h < kHold; ++h) {
+      const int z = (threadIdx.x >> ltx) + h * (blockDim.x >> ltx);
+      if (ok && z < nz) {
+        const C* at = buf + (pz.at_freq(z) << ltx) + t;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) m[h][c] = at[c * lp];
+        cs.project(m[h], sy, z, kxy0 && z == 0, free_mask);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < kHold; ++h) {
+      const int z = (threadIdx.x >> ltx) + h * (blockDim.x >> ltx);
+      if (ok && z < nz) {
+        C* at = buf + (pz.at_natural(z) << ltx) + t;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) at[c * lp] = m[h][c];
+      }
+    }
+    __syncthreads();
+    tile_dit<true, false, true>(buf, pz, ts, tw, NoIo{}, store);
   }
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kZThreads)
-    k_zproj(Cx<R>* __restrict__ spec, const GridDesc g, const int TX, const AxisPlan pz,
-            const Cx<R>* __restrict__ tw, const Cx<R>* __restrict__ gdx, const Cx<R>* __restrict__ gax,
-            const Cx<R>* __restrict__ gdy, const Cx<R>* __restrict__ gay, const Cx<R>* __restrict__ gdz,
-            const Cx<R>* __restrict__ gaz, const unsigned free_mask) {
-  zproj_body<R>(spec, g, TX, pz, tw, gdx, gax, gdy, gay, gdz, gaz, free_mask, blockIdx.x, blockIdx.y);
+__global__ void __launch_bounds__(kGZ, z_blocks<R>())
+    k_zproj(Cx<R>* __restrict__ spec, const GridDesc g, const int ltx, const __grid_constant__ AxisPlan pz,
+            const Cx<R>* __restrict__ tw, const AxisSyms<R> sy, const unsigned free_mask) {
+  zproj_body<R>(spec, g, ltx, pz, tw, sy, free_mask, blockIdx.x);
 }
 
 // ------------------------------------------------- y + projection (2D)
 template <typename R>
-__device__ __forceinline__ void yproj2d_body(Cx<R>* __restrict__ spec, const GridDesc& g, const int TX,
+__device__ __forceinline__ void yproj2d_body(Cx<R>* __restrict__ spec, const GridDesc& g, const int ltx,
                                              const AxisPlan& py, const Cx<R>* __restrict__ tw,
-                                             const Cx<R>* __restrict__ gdx, const Cx<R>* __restrict__ gax,
-                                             const Cx<R>* __restrict__ gdy, const Cx<R>* __restrict__ gay,
-                                             const unsigned free_mask, const int bx) {
+                                             const AxisSyms<R>& sy, const unsigned free_mask, const int b) {
   using C = Cx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  const int ny = g.ny, nxh = g.nxh, ncl = g.ncomp;  // lines per column: 3, or 6 for Kuhn triangles
-  const int kx0 = bx * TX;
-  const int tv = min(TX, nxh - kx0);
-  const int plane = ny * TX;
-  for (int idx = threadIdx.x; idx < ncl * plane; idx += blockDim.x) {
-    const int c = idx / plane, rem = idx - c * plane;
-    const int y = rem / TX, t = rem - y * TX;
-    buf[idx] = t < tv ? spec[((long long)c * ny + y) * nxh + kx0 + t] : C{0, 0};
-  }
-  __syncthreads();
-  const LineMap lm{TX, plane, 1, TX};
-  fft_lines<kYEpt, false, true>(buf, py, ncl * TX, lm, tw);
-  for (int pt = threadIdx.x; pt < plane; pt += blockDim.x) {
-    const int y = pt / TX, t = pt - y * TX;
-    const int kx = kx0 + t;
-    if (t >= tv) continue;
-    if (ncl == 6) {
-      C m[6];
+  const int ny = g.ny, nxh = g.nxh, ncl = g.ncomp, tx = 1 << ltx;  // 3 lines per column, or 6 (Kuhn triangles)
+  const int t = threadIdx.x & (tx - 1);
+  int zero, kx;
+  const bool ok = ColTiles(1, nxh, tx).at(b, t, &zero, &kx);
+  C* col = spec + kx;
+  auto load = [=](int c, int y, int) -> C { return ok ? col[((long long)c * ny + y) * nxh] : C{0, 0}; };
+  auto store = [=](int c, int y, int, C v) {
+    if (ok) col[((long long)c * ny + y) * nxh] = v;
+  };
+  const TileShape ts{ncl, tx, ltx};
+  tile_dit<false, true, false>(buf, py, ts, tw, load, NoIo{});
+  const int lp = py.lp << ltx;
+  if constexpr (sizeof(R) == 4) {
+    if (py.keep_order) {  // as in zproj_body
+      C m[kHold2][3];
 #pragma unroll
-      for (int c = 0; c < 6; ++c) m[c] = buf[c * plane + pt];
-      const C dx = gdx[kx], dy = gdy[y];
-      project_simplex2<R>(m, C{(R)1 + dx.x, dx.y}, dx, C{(R)1 + dy.x, dy.y}, dy, kx == 0 && y == 0, free_mask);
+      for (int h = 0; h < kHold2; ++h) {
+        const int y = (threadIdx.x >> ltx) + h * (blockDim.x >> ltx);
+        if (ok && y < ny) {
+          const C* at = buf + (py.at_freq(y) << ltx) + t;
 #pragma unroll
-      for (int c = 0; c < 6; ++c) buf[c * plane + pt] = m[c];
-      continue;
+          for (int c = 0; c < 3; ++c) m[h][c] = at[c * lp];
+          project2_at<R>(m[h], sy, kx, y, kx == 0 && y == 0, free_mask);
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int h = 0; h < kHold2; ++h) {
+        const int y = (threadIdx.x >> ltx) + h * (blockDim.x >> ltx);
+        if (ok && y < ny) {
+          C* at = buf + (py.at_natural(y) << ltx) + t;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) at[c * lp] = m[h][c];
+        }
+      }
+      __syncthreads();
+      tile_dit<true, false, true>(buf, py, ts, tw, NoIo{}, store);
+      return;
     }
-    C m[3];
+  }
+  if (ok) {
+    for (int i = threadIdx.x >> ltx; i < ny; i += blockDim.x >> ltx) {
+      const int e = py.dr[0].div(i), q0 = i - e * py.r[0], y = py.freq_of(q0, e);
+      C* at = buf + ((q0 * py.m0p + e) << ltx) + t;
+      if (ncl == 6) {
+        C m[6];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) m[c] = buf[c * plane + pt];
-    const C d0 = cmul(gdx[kx], gay[y]);
-    const C d1 = cmul(gax[kx], gdy[y]);
-    project2<R>(m, d0, d1, kx == 0 && y == 0, free_mask);
+        for (int c = 0; c < 6; ++c) m[c] = at[c * lp];
+        const C dx = sy.d[0][kx], dy = sy.d[1][y];
+        project_simplex2<R>(m, C{(R)1 + dx.x, dx.y}, dx, C{(R)1 + dy.x, dy.y}, dy, kx == 0 && y == 0, free_mask);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) buf[c * plane + pt] = m[c];
+        for (int c = 0; c < 6; ++c) at[c * lp] = m[c];
+      } else {
+        C m[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) m[c] = at[c * lp];
+        project2_at<R>(m, sy, kx, y, kx == 0 && y == 0, free_mask);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) at[c * lp] = m[c];
+      }
+    }
   }
   __syncthreads();
-  fft_lines<kYEpt, true, true>(buf, py, ncl * TX, lm, tw);
-  for (int idx = threadIdx.x; idx < ncl * plane; idx += blockDim.x) {
-    const int c = idx / plane, rem = idx - c * plane;
-    const int y = rem / TX, t = rem - y * TX;
-    if (t < tv) spec[((long long)c * ny + y) * nxh + kx0 + t] = buf[idx];
-  }
+  tile_transposed_inverse(buf, py, ts, tw, store);
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kYThreads, kXYMinBlocks)
-    k_yproj2d(Cx<R>* __restrict__ spec, const GridDesc g, const int TX, const AxisPlan py,
-              const Cx<R>* __restrict__ tw, const Cx<R>* __restrict__ gdx, const Cx<R>* __restrict__ gax,
-              const Cx<R>* __restrict__ gdy, const Cx<R>* __restrict__ gay, const unsigned free_mask) {
-  yproj2d_body<R>(spec, g, TX, py, tw, gdx, gax, gdy, gay, free_mask, blockIdx.x);
+__global__ void __launch_bounds__(kGT, xy_blocks<R>())
+    k_yproj2d(Cx<R>* __restrict__ spec, const GridDesc g, const int ltx, const __grid_constant__ AxisPlan py,
+              const Cx<R>* __restrict__ tw, const AxisSyms<R> sy, const unsigned free_mask) {
+  yproj2d_body<R>(spec, g, ltx, py, tw, sy, free_mask, blockIdx.x);
 }
 
 // ------------------------------------------------------------ x inverse
@@ -296,54 +364,65 @@ __device__ __forceinline__ void xinv_body(const Cx<R>* __restrict__ spec, R* __r
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
   __shared__ double red[32];
-  const int nx = g.nx, nc = g.ncomp, nxh = g.nxh, half = nx >> 1;
+  const int nx = g.nx, nc = g.ncomp, nxh = g.nxh, half = nx >> 1, lp = px.lp;
   const long long row0 = (long long)bx * Q;
   const int npair = (nc * Q) >> 1;
-  for (int idx = threadIdx.x; idx < npair * nx; idx += blockDim.x) {
-    const int p = idx / nx, k = idx - p * nx;
+  for (int idx = threadIdx.x; idx < npair * nxh; idx += blockDim.x) {
+    const int p = px.dh.div(idx), k = idx - p * nxh;
     C xh[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int rho = 2 * p + h;
-      const int q = rho / nc, c = rho - q * nc;
+      const int q = px.dc.div(rho), c = rho - q * nc;
       const long long row = row0 + q;
-      C x = C{0, 0};
-      if (q < Q && row < g.nrows) {
-        const int kk = k <= half ? k : nx - k;
-        x = spec[(c * g.nrows + row) * nxh + kk];
-        if (kk == 0 || kk == half) x.y = 0;
-        if (k > half) x.y = -x.y;
-      }
-      xh[h] = x;
+      xh[h] = (q < Q && row < g.nrows) ? spec[(c * g.nrows + row) * nxh + k] : C{0, 0};
+      if (k == 0 || k == half) xh[h].y = 0;
     }
-    buf[idx] = C{xh[0].x - xh[1].y, xh[0].y + xh[1].x};
+    buf[p * lp + px.at_natural(k)] = C{xh[0].x - xh[1].y, xh[0].y + xh[1].x};
+    if (k != 0 && k != half) buf[p * lp + px.at_natural(nx - k)] = C{xh[0].x + xh[1].y, xh[1].x - xh[0].y};
   }
   __syncthreads();
-  fft_lines<kXEpt, true, false>(buf, px, npair, LineMap{1, nx, 0, 1}, tw);
-  KSum<R> acc;
-  for (int idx = threadIdx.x; idx < 2 * npair * nx; idx += blockDim.x) {
-    const int rho = idx / nx, x = idx - rho * nx;
-    const int q = rho / nc, c = rho - q * nc;
-    const long long row = row0 + q;
-    if (q < Q && row < g.nrows) {
-      const C z = buf[(rho >> 1) * nx + x];
-      const R val = ((rho & 1) ? z.y : z.x) * scale;
-      const long long off = c * g.nvox + row * nx + x;
-      out[off] = val;
-      if (DOT) acc.add(val * (self_dot ? val : dotw[off]));
+  const TileShape ts{npair, 1, 0};
+  const long long nrows = g.nrows, nvox = g.nvox;
+  if constexpr (DOT) {
+    // the sums want one accumulator per thread: transform in place, then one
+    // sweep over the rows
+    tile_dit<true, false, false>(buf, px, ts, tw, NoIo{}, NoIo{});
+    KSum<R> acc;
+    for (int idx = threadIdx.x; idx < 2 * npair * nx; idx += blockDim.x) {
+      const int rho = px.dn.div(idx), x = idx - rho * nx;
+      const int q = px.dc.div(rho), c = rho - q * nc;
+      const long long row = row0 + q;
+      if (q < Q && row < nrows) {
+        const C z = buf[(rho >> 1) * lp + px.at_freq(x)];
+        const R val = ((rho & 1) ? z.y : z.x) * scale;
+        const long long off = c * nvox + row * nx + x;
+        out[off] = val;
+        acc.add(val * (self_dot ? val : dotw[off]));
+      }
     }
-  }
-  if (DOT) {
     double v[1] = {acc.value()};
     block_sum<1>(v, red);
     if (threadIdx.x == 0) *partial = v[0];
+  } else {
+    const FastDiv dc = px.dc;
+    auto store = [=](int p, int x, int, C v) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int rho = 2 * p + h;
+        const int q = dc.div(rho), c = rho - q * nc;
+        const long long row = row0 + q;
+        if (q < Q && row < nrows) out[c * nvox + row * nx + x] = (h ? v.y : v.x) * scale;
+      }
+    };
+    tile_dit<true, false, true>(buf, px, ts, tw, NoIo{}, store);
   }
 }
 
 template <typename R, bool DOT>
-__global__ void __launch_bounds__(kXThreads, kXYMinBlocks)
+__global__ void __launch_bounds__(kGT, xy_blocks<R>())
     k_xinv(const Cx<R>* __restrict__ spec, R* __restrict__ out, const R* __restrict__ dotw,
-           double* __restrict__ partials, const GridDesc g, const int Q, const AxisPlan px,
+           double* __restrict__ partials, const GridDesc g, const int Q, const __grid_constant__ AxisPlan px,
            const Cx<R>* __restrict__ tw, const R scale, const bool self_dot) {
   xinv_body<R, DOT>(spec, out, dotw, DOT ? partials + blockIdx.x : nullptr, g, Q, px, tw, scale, self_dot,
                     blockIdx.x);

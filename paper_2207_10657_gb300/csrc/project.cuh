@@ -79,6 +79,136 @@ __device__ __forceinline__ void project2(Cx<R> (&m)[3], Cx<R> d0, Cx<R> d1, bool
   m[2] = cscale(o(n0, n1, v0, v1), s2);
 }
 
+// The FP64 operator.  The symbol of the bilinear / trilinear element is
+//   D_x = (e^{i th_x} - 1) (1 + e^{i th_y})/2 (1 + e^{i th_z})/2
+//       = 2i e^{i (th_x + th_y + th_z)/2} sin(th_x/2) cos(th_y/2) cos(th_z/2)
+// (D_y, D_z alike): one complex factor common to the components times a real
+// vector s.  Ghat depends on D through D (x) D* / |D|^2 only, where the
+// common factor cancels, so it is a real operator and s (from the half-angle
+// tables) stands in for D: about 60 multiply-adds per frequency instead of
+// 150.  The FP64 passes are bound by the FP64 pipe (2 lanes per SM and clock):
+// the 128^3 product 2981 -> 2733 us.  FP32 keeps the complex form: its z
+// pass is bound elsewhere (256^3 product 1053 -> 1040 us with the real form)
+// and the FP32 solves keep their roundings.
+__device__ __forceinline__ void project3_real(double2 (&m)[6], const double s0, const double s1, const double s2,
+                                              const bool k0, const unsigned free_mask) {
+  if (k0) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+      if (!((free_mask >> c) & 1u)) m[c] = double2{0, 0};
+    return;
+  }
+  const double n2 = s0 * s0 + s1 * s1 + s2 * s2;
+  if (n2 == 0.0) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) m[c] = double2{0, 0};
+    return;
+  }
+  const double inv = 1.0 / n2, is2 = 0.70710678118654752440;
+  // v_i = sum_j zeta_ij s_j, zeta_ij = m / sqrt 2 off the diagonal
+  const double q0 = s0 * is2, q1 = s1 * is2, q2 = s2 * is2;
+  auto dot3 = [](double2 a, double x, double2 b, double y, double2 c, double z) {
+    return double2{a.x * x + b.x * y + c.x * z, a.y * x + b.y * y + c.y * z};
+  };
+  const double2 v0 = dot3(m[0], s0, m[5], q1, m[4], q2);
+  const double2 v1 = dot3(m[1], s1, m[5], q0, m[3], q2);
+  const double2 v2 = dot3(m[2], s2, m[4], q0, m[3], q1);
+  // t = -(s.v) / (2 |s|^2), w = v + t s
+  const double2 t = cscale(dot3(v0, s0, v1, s1, v2, s2), -0.5 * inv);
+  const double2 w0{v0.x + t.x * s0, v0.y + t.y * s0};
+  const double2 w1{v1.x + t.x * s1, v1.y + t.y * s1};
+  const double2 w2{v2.x + t.x * s2, v2.y + t.y * s2};
+  // 2 s / |s|^2 on the diagonal; sqrt 2 (s_i w_j + s_j w_i) / |s|^2 off it
+  const double d = 2.0 * inv, e0 = d * q0, e1 = d * q1, e2 = d * q2;
+  m[0] = cscale(w0, d * s0);
+  m[1] = cscale(w1, d * s1);
+  m[2] = cscale(w2, d * s2);
+  m[3] = double2{e1 * w2.x + e2 * w1.x, e1 * w2.y + e2 * w1.y};
+  m[4] = double2{e0 * w2.x + e2 * w0.x, e0 * w2.y + e2 * w0.y};
+  m[5] = double2{e0 * w1.x + e1 * w0.x, e0 * w1.y + e1 * w0.y};
+}
+
+// 2D: s_x = sin(th_x/2) cos(th_y/2), s_y = cos(th_x/2) sin(th_y/2).
+__device__ __forceinline__ void project2_real(double2 (&m)[3], const double s0, const double s1, const bool k0,
+                                              const unsigned free_mask) {
+  if (k0) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (!((free_mask >> c) & 1u)) m[c] = double2{0, 0};
+    return;
+  }
+  const double n2 = s0 * s0 + s1 * s1;
+  if (n2 == 0.0) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) m[c] = double2{0, 0};
+    return;
+  }
+  const double inv = 1.0 / n2, is2 = 0.70710678118654752440, q0 = s0 * is2, q1 = s1 * is2;
+  const double2 v0{m[0].x * s0 + m[2].x * q1, m[0].y * s0 + m[2].y * q1};
+  const double2 v1{m[1].x * s1 + m[2].x * q0, m[1].y * s1 + m[2].y * q0};
+  const double2 t = cscale(double2{v0.x * s0 + v1.x * s1, v0.y * s0 + v1.y * s1}, -0.5 * inv);
+  const double2 w0{v0.x + t.x * s0, v0.y + t.y * s0};
+  const double2 w1{v1.x + t.x * s1, v1.y + t.y * s1};
+  const double d = 2.0 * inv, e0 = d * q0, e1 = d * q1;
+  m[0] = cscale(w0, d * s0);
+  m[1] = cscale(w1, d * s1);
+  m[2] = double2{e0 * w1.x + e1 * w0.x, e0 * w1.y + e1 * w0.y};
+}
+
+// Symbol tables of the axes: d[a][k] = e^{i th} - 1 (exact 0 at k = 0);
+// h[a][k] = (1 + e^{i th}) / 2 (exact 0 at 2k = n) in FP32, the half-angle
+// pair (sin(th/2), cos(th/2)) in FP64 (exact 0 at k = 0 / 2k = n).
+template <typename R> struct AxisSyms {
+  const Cx<R>* d[3];
+  const Cx<R>* h[3];
+};
+
+// The x and y factors of a column's symbol, formed once; project() applies
+// Ghat at z frequency kz.
+template <typename R> struct ColSym3;
+template <> struct ColSym3<float> {
+  float2 ay, dy;
+  int kx;
+  __device__ __forceinline__ ColSym3() {}
+  __device__ __forceinline__ ColSym3(const AxisSyms<float>& s, int kx_, int ky) : ay(s.h[1][ky]), dy(s.d[1][ky]), kx(kx_) {}
+  __device__ __forceinline__ void project(float2 (&m)[6], const AxisSyms<float>& s, int kz, bool k0,
+                                          unsigned free_mask) const {
+    const float2 ax = s.h[0][kx], dx = s.d[0][kx], az = s.h[2][kz], dz = s.d[2][kz];
+    const float2 d0 = cmul(cmul(dx, ay), az);
+    const float2 d1 = cmul(cmul(ax, dy), az);
+    const float2 d2 = cmul(cmul(ax, ay), dz);
+    project3<float>(m, d0, d1, d2, k0, free_mask);
+  }
+};
+template <> struct ColSym3<double> {
+  double fx, fy, fz;
+  __device__ __forceinline__ ColSym3() {}
+  __device__ __forceinline__ ColSym3(const AxisSyms<double>& s, int kx, int ky) {
+    const double2 hx = s.h[0][kx], hy = s.h[1][ky];
+    fx = hx.x * hy.y;
+    fy = hx.y * hy.x;
+    fz = hx.y * hy.y;
+  }
+  __device__ __forceinline__ void project(double2 (&m)[6], const AxisSyms<double>& s, int kz, bool k0,
+                                          unsigned free_mask) const {
+    const double2 hz = s.h[2][kz];
+    project3_real(m, fx * hz.y, fy * hz.y, fz * hz.x, k0, free_mask);
+  }
+};
+
+template <typename R>
+__device__ __forceinline__ void project2_at(Cx<R> (&m)[3], const AxisSyms<R>& s, int kx, int ky, bool k0,
+                                            unsigned free_mask) {
+  if constexpr (sizeof(R) == 4) {
+    const float2 d0 = cmul(s.d[0][kx], s.h[1][ky]);
+    const float2 d1 = cmul(s.h[0][kx], s.d[1][ky]);
+    project2<float>(m, d0, d1, k0, free_mask);
+  } else {
+    const double2 hx = s.h[0][kx], hy = s.h[1][ky];
+    project2_real(m, hx.x * hy.y, hx.y * hy.x, k0, free_mask);
+  }
+}
+
 // Ghat(k) for the 2D Kuhn-triangle discretisation (every pixel split along
 // its main diagonal into two linear triangles, one strain each; Sec. 2.1
 // builds the projection from any FE gradient).  m holds the six lines
