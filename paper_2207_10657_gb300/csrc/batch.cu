@@ -29,7 +29,10 @@ using R = float;
 using C = float2;
 
 constexpr int kMaxBatch = 256;
-constexpr int kXYPerSM = 8;               // blocks per SM of the x / y / 2D launches
+// resident blocks per SM of the x / y / 2D launches: the items' starts are
+// latency, so two more blocks than the single-grid kernels pay here (96 cells
+// 2.87 -> 2.70 ms; a single 160x120x90 grid 199 -> 206 us)
+constexpr int kXYPerSM = 8;
 constexpr long long kVecChunk = 16384;  // field elements per vector item (multiple of 4)
 constexpr long long kVoxChunk = 4096;   // voxels per constitutive item (multiple of 4)
 
@@ -73,47 +76,93 @@ struct WLists {
   int start[BP_N][kMaxBatch + 1];     // item prefix over active members
 };
 
-// Pull the next item of pass `pass`; false when exhausted.  Uniform across
-// the block.  *v is the item's index (also its partial-sum slot).
-__device__ __forceinline__ bool fetch(const WLists* __restrict__ wl, int pass, int* counter, int* s_item, int* v,
-                                      int* member, int* local) {
-  __syncthreads();
-  if (threadIdx.x == 0) *s_item = atomicAdd(counter, 1);
-  __syncthreads();
-  const int it = *s_item;
-  if (it >= wl->total[pass]) return false;
-  const int* st = wl->start[pass];
-  int lo = 0, hi = wl->count - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (st[mid] <= it) lo = mid;
-    else hi = mid - 1;
-  }
-  *v = it;
-  *member = wl->idx[lo];
-  *local = it - st[lo];
-  return true;
-}
+// A block's view of one pass's work list: the prefixes and member ids of the
+// active members, copied to shared memory once, and the next item's number,
+// asked for an item ahead (the counter's round trip runs behind the current
+// item's work).  Per item this leaves two barriers and a search in shared
+// memory; with the counter and the search in global memory an item began
+// with a chain of eight dependent loads.
+struct ItemQueue {
+  int* sh;       // kItemWords ints of shared memory
+  int* counter;
+  int next;      // thread 0: the next item
+  int count, total;
 
-// One block: the members passing the gate, in order, and their item
-// prefixes for every pass (nb: BP_N x n block counts).
-__global__ void kb_compact(WLists* wl, const int* __restrict__ nb, int n, Gate gt, const DevScalars* S) {
-  __shared__ int flag[kMaxBatch];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) flag[i] = gate_ok(gt, S, i) ? 1 : 0;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int k = 0;
-    for (int i = 0; i < n; ++i)
-      if (flag[i]) wl->idx[k++] = i;
-    wl->count = k;
-    for (int p = 0; p < BP_N; ++p) {
-      int sum = 0;
-      for (int q = 0; q < k; ++q) {
-        wl->start[p][q] = sum;
-        sum += nb[p * n + wl->idx[q]];
-      }
-      wl->start[p][k] = sum;
-      wl->total[p] = sum;
+  static constexpr int kItemWords = 2 * kMaxBatch + 2;
+
+  __device__ __forceinline__ ItemQueue(int* sh_, const WLists* __restrict__ wl, int pass, int* counter_)
+      : sh(sh_), counter(counter_), next(0), count(wl->count), total(wl->total[pass]) {
+    if (threadIdx.x == 0) next = atomicAdd(counter, 1);
+    for (int k = threadIdx.x; k < count; k += blockDim.x) {
+      sh[k] = wl->start[pass][k];
+      sh[kMaxBatch + k] = wl->idx[k];
+    }
+  }
+  // Next item; false when exhausted.  Uniform across the block.  *v is the
+  // item's index (also its partial-sum slot).
+  __device__ __forceinline__ bool fetch(int* v, int* member, int* local) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      sh[2 * kMaxBatch] = next;
+      if (next < total) next = atomicAdd(counter, 1);
+    }
+    __syncthreads();
+    const int it = sh[2 * kMaxBatch];
+    if (it >= total) return false;
+    int lo = 0, hi = count - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (sh[mid] <= it) lo = mid;
+      else hi = mid - 1;
+    }
+    *v = it;
+    *member = sh[kMaxBatch + lo];
+    *local = it - sh[lo];
+    return true;
+  }
+};
+
+// One block of kMaxBatch threads: the members passing the gate, in order, and
+// their item prefixes for every pass (nb: BP_N x n block counts), by scans
+// over the block (one thread doing it took 45 us for 96 members, three times
+// per CG iteration; now 4 us).
+__global__ void __launch_bounds__(kMaxBatch)
+    kb_compact(WLists* wl, const int* __restrict__ nb, int n, Gate gt, const DevScalars* S) {
+  __shared__ int wsum[kMaxBatch / 32];
+  const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
+  // inclusive sum of x over the threads 0 .. i; *all: over the block
+  auto scan = [&](int x, int* all) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    int before = 0, sum = 0;
+#pragma unroll
+    for (int w = 0; w < kMaxBatch / 32; ++w) {
+      if (w < warp) before += wsum[w];
+      sum += wsum[w];
+    }
+    *all = sum;
+    return before + x;
+  };
+  const int on = i < n && gate_ok(gt, S, i) ? 1 : 0;
+  int count;
+  const int k = scan(on, &count) - on;  // this member's place among the active ones
+  if (on) wl->idx[k] = i;
+  if (i == 0) wl->count = count;
+#pragma unroll
+  for (int p = 0; p < BP_N; ++p) {
+    const int x = on ? nb[p * n + i] : 0;
+    int total;
+    const int end = scan(x, &total);
+    if (on) wl->start[p][k] = end - x;
+    if (i == 0) {
+      wl->start[p][count] = total;
+      wl->total[p] = total;
     }
   }
 }
@@ -129,36 +178,46 @@ __device__ __forceinline__ const BDesc& member_desc(const BDesc* d, int* s) {
 }
 
 // ------------------------------------------------------ spectral passes
-// XMODE: 0 plain x-forward, 1 tangent x-forward.  YINV: y direction.
+// The members' own fields (rve_batch_hessp), read and written in place: with
+// a copy per member in and out, the 192 copies of a 96-member product took
+// 1.6 of its 4.6 ms.
+struct MemberFields {
+  R* p[kMaxBatch];
+};
+
+// XMODE: 0 plain x-forward, 1 tangent, 2 consistent tangent.  YINV: y direction.  EXT: the
+// input / output is the members' own fields instead of the batched vector.
 // DOT for the x-inverse: 0 none, 1 with dotw, 2 self.
 // cdp, ca, cn (batched like the state, may be NULL): the rank-one part of
-// the symmetric consistent tangent (ConsTan), applied with XMODE 1.
-template <int XMODE>
-__global__ void __launch_bounds__(kGT, xy_blocks<R>())
+// the symmetric consistent tangent (ConsTan), applied with XMODE 2.
+template <int XMODE, bool EXT>
+__global__ void __launch_bounds__(kGT, kXYPerSM)
     kb_xfwd(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter,
             const DevScalars* __restrict__ S, const MatTable<R> mt, const R* __restrict__ in,
             const uint8_t* __restrict__ phase, const R* __restrict__ dmg, const R* __restrict__ cdp,
-            const R* __restrict__ ca, const R* __restrict__ cn) {
-  __shared__ int s_item;
+            const R* __restrict__ ca, const R* __restrict__ cn, const __grid_constant__ MemberFields ext) {
+  __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
+  ItemQueue items(s_items, wl, BP_X, counter);
   for (;;) {
     int v, i, lb;
-    if (!fetch(wl, BP_X, counter, &s_item, &v, &i, &lb)) break;
+    if (!items.fetch(&v, &i, &lb)) break;
     const BDesc& d = member_desc(D + i, s_desc);
-    const ConsTan<R> ct{cdp ? cdp + d.voff : nullptr, ca ? ca + d.foff : nullptr, cn ? cn + d.foff : nullptr};
-    xfwd_body<R, XMODE>(in + d.foff, phase + d.voff, dmg + d.voff, mt, d.spec, d.g, d.qx, d.px, d.tw[0],
+    const ConsTan<R> ct = XMODE == 2 ? ConsTan<R>{cdp + d.voff, ca + d.foff, cn + d.foff} : ConsTan<R>{};
+    xfwd_body<R, XMODE>(EXT ? ext.p[i] : in + d.foff, phase + d.voff, dmg + d.voff, mt, d.spec, d.g, d.qx, d.px, d.tw[0],
                         lb, ct);
   }
 }
 
 template <bool YINV>
-__global__ void __launch_bounds__(kGT, xy_blocks<R>())
+__global__ void __launch_bounds__(kGT, kXYPerSM)
     kb_ycols(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter) {
-  __shared__ int s_item;
+  __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
+  ItemQueue items(s_items, wl, BP_Y, counter);
   for (;;) {
     int v, i, lb;
-    if (!fetch(wl, BP_Y, counter, &s_item, &v, &i, &lb)) break;
+    if (!items.fetch(&v, &i, &lb)) break;
     const BDesc& d = member_desc(D + i, s_desc);
     ycols_body<R, YINV>(d.spec, d.g, d.lty, d.py, d.tw[1], lb);
   }
@@ -166,41 +225,44 @@ __global__ void __launch_bounds__(kGT, xy_blocks<R>())
 
 __global__ void __launch_bounds__(kGZ, z_blocks<R>())
     kb_zproj(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter) {
-  __shared__ int s_item;
+  __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
+  ItemQueue items(s_items, wl, BP_Z, counter);
   for (;;) {
     int v, i, lb;
-    if (!fetch(wl, BP_Z, counter, &s_item, &v, &i, &lb)) break;
+    if (!items.fetch(&v, &i, &lb)) break;
     const BDesc& d = member_desc(D + i, s_desc);
     zproj_body<R>(d.spec, d.g, d.ltz, d.pz, d.tw[2], d.sy, d.free_mask, lb);
   }
 }
 
-__global__ void __launch_bounds__(kGT, xy_blocks<R>())
+__global__ void __launch_bounds__(kGT, kXYPerSM)
     kb_yproj2d(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter) {
-  __shared__ int s_item;
+  __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
+  ItemQueue items(s_items, wl, BP_2D, counter);
   for (;;) {
     int v, i, lb;
-    if (!fetch(wl, BP_2D, counter, &s_item, &v, &i, &lb)) break;
+    if (!items.fetch(&v, &i, &lb)) break;
     const BDesc& d = member_desc(D + i, s_desc);
     yproj2d_body<R>(d.spec, d.g, d.ltz, d.py, d.tw[1], d.sy, d.free_mask, lb);
   }
 }
 
-template <int DOT>
-__global__ void __launch_bounds__(kGT, xy_blocks<R>())
+template <int DOT, bool EXT>
+__global__ void __launch_bounds__(kGT, kXYPerSM)
     kb_xinv(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter,
             const DevScalars* __restrict__ S, R* __restrict__ out, const R* __restrict__ dotw,
-            double* __restrict__ partials) {
-  __shared__ int s_item;
+            double* __restrict__ partials, const __grid_constant__ MemberFields ext) {
+  __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
+  ItemQueue items(s_items, wl, BP_X, counter);
   for (;;) {
     int v, i, lb;
-    if (!fetch(wl, BP_X, counter, &s_item, &v, &i, &lb)) break;
+    if (!items.fetch(&v, &i, &lb)) break;
     const BDesc& d = member_desc(D + i, s_desc);
     const R scale = (R)(1.0 / (double)d.g.nvox);
-    xinv_body<R, DOT != 0>(d.spec, out + d.foff, DOT == 1 ? dotw + d.foff : nullptr,
+    xinv_body<R, DOT != 0>(d.spec, EXT ? ext.p[i] : out + d.foff, DOT == 1 ? dotw + d.foff : nullptr,
                            DOT ? partials + v : nullptr, d.g, d.qx, d.px, d.tw[0], scale, DOT == 2, lb);
   }
 }
@@ -234,11 +296,12 @@ __global__ void __launch_bounds__(256)
            DevScalars* __restrict__ S, R* __restrict__ a, R* __restrict__ b, R* __restrict__ c,
            const R* __restrict__ x, const R* __restrict__ y, const double* __restrict__ dE6,
            double* __restrict__ part) {
-  __shared__ int s_item;
+  __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ double red[NS > 0 ? NS * 32 : 32];
+  ItemQueue items(s_items, wl, BP_VEC, counter);
   for (;;) {
     int v, i, lb;
-    if (!fetch(wl, BP_VEC, counter, &s_item, &v, &i, &lb)) break;
+    if (!items.fetch(&v, &i, &lb)) break;
     const BDesc& d = D[i];
     const long long nf = (long long)d.g.ncomp * d.g.nvox;
     const long long e0 = (long long)(lb) * kVecChunk;
@@ -307,10 +370,11 @@ __global__ void __launch_bounds__(256)
 __global__ void __launch_bounds__(256)
     kb_scopy(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter, R* __restrict__ a,
              const R* __restrict__ x) {
-  __shared__ int s_item;
+  __shared__ int s_items[ItemQueue::kItemWords];
+  ItemQueue items(s_items, wl, BP_VOX, counter);
   for (;;) {
     int v, i, lb;
-    if (!fetch(wl, BP_VOX, counter, &s_item, &v, &i, &lb)) break;
+    if (!items.fetch(&v, &i, &lb)) break;
     const BDesc& d = D[i];
     const long long v0 = (long long)(lb) * kVoxChunk;
     const long long v1 = min(d.g.nvox, v0 + kVoxChunk);
@@ -329,12 +393,13 @@ __global__ void __launch_bounds__(256)
              const R* __restrict__ sig0, const R* __restrict__ D0, R* __restrict__ sig_t, R* __restrict__ D_t,
              R* __restrict__ kap_t, double* __restrict__ part, const R* __restrict__ cdp = nullptr,
              const R* __restrict__ ca = nullptr, const R* __restrict__ cn = nullptr) {
-  __shared__ int s_item;
+  __shared__ int s_items[ItemQueue::kItemWords];
   constexpr int NS = MEANS ? 12 : 6;
   __shared__ double red[NS * 32];
+  ItemQueue items(s_items, wl, BP_VOX, counter);
   for (;;) {
     int v, i, lb;
-    if (!fetch(wl, BP_VOX, counter, &s_item, &v, &i, &lb)) break;
+    if (!items.fetch(&v, &i, &lb)) break;
     const BDesc& d = D[i];
     const int nc = d.g.ncomp, nd = d.g.ndim;
     const long long nv = d.g.nvox;
@@ -548,7 +613,7 @@ cudaError_t reset_counters(rve_batch_ctx* c) {
 }
 
 cudaError_t compact(rve_batch_ctx* c, Gate gt) {
-  kb_compact<<<1, 256, 0, c->st>>>(c->wl, c->dnb, c->n, gt, c->S);
+  kb_compact<<<1, kMaxBatch, 0, c->st>>>(c->wl, c->dnb, c->n, gt, c->S);
   ++c->launches;
   return cudaGetLastError();
 }
@@ -562,8 +627,10 @@ cudaError_t seg_reduce(rve_batch_ctx* c, int pass, int ns, size_t off) {
 
 // Hessian-vector product (tangent) or projection (plain) of every gated RVE:
 // out = G : (B : in) or G : in; with dot, sum(out * dotw) (or |out|^2 when
-// dotw == out) into DevScalars at byte offset dot_off.
-cudaError_t batch_apply(rve_batch_ctx* c, const R* in, R* out, bool tangent, const R* dotw, size_t dot_off, Gate gt) {
+// dotw == out) into DevScalars at byte offset dot_off.  ein / eout (tangent, no
+// dot): the members' own fields instead of the batched vectors in / out.
+cudaError_t batch_apply(rve_batch_ctx* c, const R* in, R* out, bool tangent, const R* dotw, size_t dot_off, Gate gt,
+                        const MemberFields* ein = nullptr, const MemberFields* eout = nullptr) {
   cudaError_t e;
   if ((e = compact(c, gt)) != cudaSuccess) return e;
   {
@@ -572,13 +639,21 @@ cudaError_t batch_apply(rve_batch_ctx* c, const R* in, R* out, bool tangent, con
     // rank-one part of the current state (refreshed whenever eps or the
     // history change), also inside the captured CG graphs
     const bool cons = c->cdp != nullptr;
-    if (tangent)
-      kb_xfwd<1><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(
-          c->dD, c->wl, next_counter(c), c->S, c->mt, in, c->phase, c->D, cons ? c->cdp : nullptr,
-          cons ? c->ca : nullptr, cons ? c->cn : nullptr);
-    else
-      kb_xfwd<0><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(
-          c->dD, c->wl, next_counter(c), c->S, c->mt, in, c->phase, c->D, nullptr, nullptr, nullptr);
+    const MemberFields none{};
+    auto launch = [&](auto kernel) {
+      kernel<<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S, c->mt, in,
+                                                                     c->phase, c->D, c->cdp, c->ca, c->cn,
+                                                                     ein ? *ein : none);
+    };
+    if (ein) {
+      if (cons) launch(kb_xfwd<2, true>);
+      else launch(kb_xfwd<1, true>);
+    } else if (tangent) {
+      if (cons) launch(kb_xfwd<2, false>);
+      else launch(kb_xfwd<1, false>);
+    } else {
+      launch(kb_xfwd<0, false>);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (c->any3d) {
@@ -597,19 +672,19 @@ cudaError_t batch_apply(rve_batch_ctx* c, const R* in, R* out, bool tangent, con
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const int tot = c->total[BP_X];
-  if (!dotw) {
-    kb_xinv<0><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl,
-                                                                      next_counter(c), c->S, out, nullptr,
-                                                                      nullptr);
-  } else if (dotw == out) {
-    kb_xinv<2><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl,
-                                                                      next_counter(c), c->S, out, nullptr,
-                                                                      c->part);
-  } else {
-    kb_xinv<1><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl,
-                                                                      next_counter(c), c->S, out, dotw,
-                                                                      c->part);
-  }
+  const MemberFields none{};
+  if (eout)
+    kb_xinv<0, true><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S,
+                                                                             nullptr, nullptr, nullptr, *eout);
+  else if (!dotw)
+    kb_xinv<0, false><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S, out,
+                                                                              nullptr, nullptr, none);
+  else if (dotw == out)
+    kb_xinv<2, false><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S, out,
+                                                                              nullptr, c->part, none);
+  else
+    kb_xinv<1, false><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S, out,
+                                                                              dotw, c->part, none);
   c->launches += 2;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (dotw) return seg_reduce(c, BP_X, 1, dot_off);
@@ -1043,11 +1118,15 @@ rve_status batch_init(rve_batch_ctx* c, const int* dims, const int* ndims, const
   BCK(cudaMemsetAsync(c->khist, 0, vb, c->st), "memset");
   BCK(cudaMemsetAsync(c->kap, 0, vb, c->st), "memset");
   // kernel attributes for the largest dynamic shared memory
-  BCK((cudaFuncSetAttribute(kb_xfwd<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
-  BCK((cudaFuncSetAttribute(kb_xfwd<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
-  BCK((cudaFuncSetAttribute(kb_xinv<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
-  BCK((cudaFuncSetAttribute(kb_xinv<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
-  BCK((cudaFuncSetAttribute(kb_xinv<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
+  BCK((cudaFuncSetAttribute(kb_xfwd<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
+  BCK((cudaFuncSetAttribute(kb_xfwd<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
+  BCK((cudaFuncSetAttribute(kb_xfwd<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
+  BCK((cudaFuncSetAttribute(kb_xfwd<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
+  BCK((cudaFuncSetAttribute(kb_xfwd<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
+  BCK((cudaFuncSetAttribute(kb_xinv<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
+  BCK((cudaFuncSetAttribute(kb_xinv<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
+  BCK((cudaFuncSetAttribute(kb_xinv<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
+  BCK((cudaFuncSetAttribute(kb_xinv<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
   BCK((cudaFuncSetAttribute(kb_ycols<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
   BCK((cudaFuncSetAttribute(kb_ycols<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
   BCK((cudaFuncSetAttribute(kb_zproj, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap)), "attr");
@@ -1223,18 +1302,18 @@ rve_status rve_batch_solve_step(rve_batch_t c, const double* dE, const uint8_t* 
 rve_status rve_batch_hessp(rve_batch_t c, const float* const* v_dev, float* const* out_dev) {
   if (!c) return RVE_ERR_ARG;
   if (!v_dev || !out_dev) return bfail(c, RVE_ERR_ARG, "NULL argument");
+  MemberFields vin{}, vout{};
   for (int i = 0; i < c->n; ++i) {
-    const size_t b = (size_t)c->g[i].ncomp * c->g[i].nvox * sizeof(R);
-    BCK(cudaMemcpyAsync(c->d + c->desc[i].foff, v_dev[i], b, cudaMemcpyDeviceToDevice, c->st), "input copy");
+    if (!v_dev[i] || !out_dev[i]) return bfail(c, RVE_ERR_ARG, "NULL member field");
+    vin.p[i] = const_cast<R*>(v_dev[i]);
+    vout.p[i] = out_dev[i];
   }
+  // every input is read (by the x-forward launch) before any output is
+  // written (by the x-inverse launch): the fields may alias
   std::vector<char> all(c->n, 1);
   BCK(reset_counters(c), "memset");
-  BCK(batch_apply(c, c->d, c->Hd, true, nullptr, 0, gate_bits(all)), "hessp");
+  BCK(batch_apply(c, nullptr, nullptr, true, nullptr, 0, gate_bits(all), &vin, &vout), "hessp");
   c->hv += c->n;
-  for (int i = 0; i < c->n; ++i) {
-    const size_t b = (size_t)c->g[i].ncomp * c->g[i].nvox * sizeof(R);
-    BCK(cudaMemcpyAsync(out_dev[i], c->Hd + c->desc[i].foff, b, cudaMemcpyDeviceToDevice, c->st), "output copy");
-  }
   return RVE_OK;
 }
 

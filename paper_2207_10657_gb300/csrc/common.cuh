@@ -31,6 +31,13 @@ template <bool INV, typename C> __device__ __forceinline__ C rot90(C a) {
 
 constexpr int kMaxPhases = 16;
 
+// single-rounding product and fused multiply-add: where the result must not
+// depend on which product of a sum the compiler contracts
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // ------------------------------------------------------ radix butterflies
 // Small DFTs with the constants of the R-th roots of unity written out.
 template <int R, bool INV, typename C> struct Dft;

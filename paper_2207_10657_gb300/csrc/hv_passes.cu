@@ -143,7 +143,7 @@ GenericTiles<R>::GenericTiles(const GridDesc& g, int qx, int lty, int ltz, const
                               const AxisPlan& pz) {
   using C = Cx<R>;
   xblocks = (int)((g.nrows + qx - 1) / qx);
-  xsmem = (size_t)((g.ncomp * qx) / 2) * px.lp * sizeof(C);
+  xsmem = (size_t)((g.ncomp * qx) / 2) * px.lp * sizeof(C) + XTables::bytes((g.ncomp * qx) / 2, g.nx);
   if (g.ndim == 3) {
     yblocks = ColTiles(g.ncomp * g.nz, g.nxh, 1 << lty).count();
     ysmem = (size_t)(py.lp << lty) * sizeof(C);
@@ -195,6 +195,7 @@ cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w) {
   // opt in to large dynamic shared memory
   cudaFuncSetAttribute(k_xfwd<R, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
   cudaFuncSetAttribute(k_xfwd<R, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
+  cudaFuncSetAttribute(k_xfwd<R, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
   cudaFuncSetAttribute(k_ycols<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
   cudaFuncSetAttribute(k_ycols<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
   cudaFuncSetAttribute(k_zproj<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
@@ -343,7 +344,9 @@ cudaError_t spectral_apply(const GridDesc& g, SpecWork<R>& w, const MatTable<R>&
     }
   }
   if (e == cudaErrorNotSupported) {
-    if (mode == XIn::Tangent)
+    if (mode == XIn::Tangent && w.cons.dp)
+      k_xfwd<R, 2><<<xblocks, kGT, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0], w.cons);
+    else if (mode == XIn::Tangent)
       k_xfwd<R, 1><<<xblocks, kGT, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0], w.cons);
     else
       k_xfwd<R, 0><<<xblocks, kGT, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0],
