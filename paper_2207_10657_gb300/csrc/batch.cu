@@ -1033,6 +1033,7 @@ rve_status batch_init(rve_batch_ctx* c, const int* dims, const int* ndims, const
     g.ny = dims[3 * i + 1];
     g.nz = g.ndim == 3 ? dims[3 * i + 2] : 1;
     g.nxh = g.nx / 2 + 1;
+    g.nxs = spectrum_stride(g.nxh);
     g.ncomp = g.ndim == 3 ? 6 : 3;
     g.nvox = (long long)g.nx * g.ny * g.nz;
     g.nrows = (long long)g.ny * g.nz;

@@ -213,7 +213,7 @@ cudaError_t spectral_setup(const GridDesc& g, SpecWork<R>& w) {
   const int ns[3] = {g.nx, g.ny, g.nz};
   for (int a = 0; a < g.ndim; ++a)
     if ((e = upload_tables<R>(ns[a], &w.tw[a], &w.gdiff[a], &w.gavg[a])) != cudaSuccess) return e;
-  const size_t nspec = (size_t)g.ncomp * g.nrows * g.nxh;
+  const size_t nspec = (size_t)g.ncomp * g.nrows * g.nxs;
   if ((e = cudaMalloc(&w.spec, nspec * sizeof(C))) != cudaSuccess) return e;
   if (std::is_same<R, float>::value && cluster_size_ok(g)) {
     // twiddles of the cluster passes' M-point y sub-transform (M = Nx / 4)

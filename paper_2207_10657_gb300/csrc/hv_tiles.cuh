@@ -56,7 +56,7 @@ template <int N, int NROW> struct RowItems {
 // ------------------------------------------------------------ x forward
 template <int N, int NC>
 __device__ __forceinline__ void xfwd_fft_store(float2* buf, float2* __restrict__ spec, const long long nrows,
-                                               const float2* __restrict__ tw, const long long row0,
+                                               const int nxs, const float2* __restrict__ tw, const long long row0,
                                                const long long row_end);
 
 // One x-forward tile: the voxel rows [row0, row_end) (at most xq rows),
@@ -69,7 +69,7 @@ template <int N, int NC, int MODE>
 __device__ __forceinline__ float xfwd_rows(float2* buf, const float* __restrict__ in,
                                            const uint8_t* __restrict__ phase, const float* __restrict__ dmg,
                                            const MatTable<float>& mt, float2* __restrict__ spec,
-                                           const long long nrows, const long long nvox,
+                                           const long long nrows, const int nxs, const long long nvox,
                                            const float2* __restrict__ tw, const long long row0,
                                            const long long row_end, const float* __restrict__ cdp,
                                            const float* __restrict__ ca, const float* __restrict__ cn) {
@@ -157,7 +157,7 @@ __device__ __forceinline__ float xfwd_rows(float2* buf, const float* __restrict_
     }
   }
   __syncthreads();
-  xfwd_fft_store<N, NC>(buf, spec, nrows, tw, row0, row_end);
+  xfwd_fft_store<N, NC>(buf, spec, nrows, nxs, tw, row0, row_end);
   return acc;
 }
 
@@ -171,14 +171,13 @@ __device__ __forceinline__ float xfwd_rows(float2* buf, const float* __restrict_
 // alone, so no per-item division by the half-spectrum length.
 template <int N, int NC>
 __device__ __forceinline__ void xfwd_fft_store(float2* buf, float2* __restrict__ spec, const long long nrows,
-                                               const float2* __restrict__ tw, const long long row0,
+                                               const int nxs, const float2* __restrict__ tw, const long long row0,
                                                const long long row_end) {
   constexpr int Q = xq<N, NC>();
   constexpr int NL = NC * Q / 2;
   fft_ct<N, NL, kFT, false>(buf, tw);
-  constexpr int NXH = N / 2 + 1;
   constexpr int KB = N / 2, GB = kFT / KB, JB = (NL + GB - 1) / GB;
-  const long long plane = nrows * NXH;
+  const long long plane = nrows * nxs;
   {
     const int g = threadIdx.x / KB, k = threadIdx.x - (threadIdx.x / KB) * KB;
     const int km = k == 0 ? 0 : N - k;
@@ -194,7 +193,7 @@ __device__ __forceinline__ void xfwd_fft_store(float2* buf, float2* __restrict__
           for (int h = 0; h < 2; ++h) {
             const int rho = 2 * p + h;
             const int q = rho / NC, c = rho - (rho / NC) * NC;
-            if (row0 + q < row_end) spec[c * plane + (row0 + q) * NXH + k] = h ? xb : xa;
+            if (row0 + q < row_end) spec[c * plane + (row0 + q) * nxs + k] = h ? xb : xa;
           }
         }
       }
@@ -206,7 +205,7 @@ __device__ __forceinline__ void xfwd_fft_store(float2* buf, float2* __restrict__
       for (int h = 0; h < 2; ++h) {
         const int rho = 2 * p + h;
         const int q = rho / NC, c = rho - (rho / NC) * NC;
-        if (row0 + q < row_end) spec[c * plane + (row0 + q) * NXH + KB] = make_float2(h ? z.y : z.x, 0.f);
+        if (row0 + q < row_end) spec[c * plane + (row0 + q) * nxs + KB] = make_float2(h ? z.y : z.x, 0.f);
       }
     }
   }
@@ -226,21 +225,20 @@ template <int N, int NC, bool DOT, bool CG, bool L2LOAD>
 __device__ __forceinline__ void xinv_rows(float2* buf, double* red, const float2* __restrict__ spec,
                                           float* __restrict__ out, const float* __restrict__ dotw,
                                           double* __restrict__ partials, const long long nrows,
-                                          const long long nvox, const float2* __restrict__ tw, const float scale,
+                                          const int nxs, const long long nvox, const float2* __restrict__ tw, const float scale,
                                           const bool self_dot, float* __restrict__ cz, float* __restrict__ cr,
                                           const float* __restrict__ cd, const int* __restrict__ cstatus,
                                           const double* __restrict__ calpha, const double* __restrict__ ctau,
                                           const long long row0, const long long row_end, const long long pidx) {
   constexpr int Q = xq<N, NC>();
   constexpr int NL = NC * Q / 2;
-  constexpr int NXH = N / 2 + 1;
   // Each half-spectrum entry kk of the two real rows packed in line p is read
   // once and fills both buf[kk] and buf[N - kk] (Hermitian symmetry).
   // Thread t takes bin kk = t mod (N/2) of the lines p = t div (N/2) + j
   // (256 / (N/2)), all its loads issued before its stores; the Nyquist bin of
   // every line goes to threads 0 .. NL-1.
   constexpr int KB = N / 2, GB = kFT / KB, JB = (NL + GB - 1) / GB;
-  const long long plane = nrows * NXH;
+  const long long plane = nrows * nxs;
   {
     const int g = threadIdx.x / KB, kk = threadIdx.x - (threadIdx.x / KB) * KB;
     if (g < GB) {
@@ -252,7 +250,7 @@ __device__ __forceinline__ void xinv_rows(float2* buf, double* red, const float2
         for (int h = 0; h < 2; ++h) {
           const int rho = 2 * p + h;
           const int q = rho / NC, c = rho - (rho / NC) * NC;
-          const float2* src = spec + c * plane + (row0 + q) * NXH + kk;
+          const float2* src = spec + c * plane + (row0 + q) * nxs + kk;
           xh[j][h] = ((JB * GB == NL || p < NL) && row0 + q < row_end) ? (L2LOAD ? __ldcg(src) : *src)
                                                                        : make_float2(0.f, 0.f);
         }
@@ -278,7 +276,7 @@ __device__ __forceinline__ void xinv_rows(float2* buf, double* red, const float2
       for (int h = 0; h < 2; ++h) {
         const int rho = 2 * p + h;
         const int q = rho / NC, c = rho - (rho / NC) * NC;
-        const float2* src = spec + c * plane + (row0 + q) * NXH + KB;
+        const float2* src = spec + c * plane + (row0 + q) * nxs + KB;
         xn[h] = row0 + q < row_end ? (L2LOAD ? __ldcg(src) : *src) : make_float2(0.f, 0.f);
       }
       buf[KB * NL + p] = make_float2(xn[0].x, xn[1].x);  // imaginary parts of the Nyquist bin dropped
@@ -367,22 +365,18 @@ __device__ __forceinline__ void xinv_rows(float2* buf, double* red, const float2
 }
 
 // ------------------------------------------------------------ y columns
-// One y tile: columns [kx0, kx0 + ytx) of the plane whose first row is
-// `plane` (row index (c Nz + z) Ny), transformed in place.  L2LOAD as for
-// xinv_rows.
-template <int N, bool INV, bool L2LOAD>
-__device__ __forceinline__ void ycols_tile(float2* buf, float2* __restrict__ spec, const long long plane,
-                                           const int kx0, const int nxh, const float2* __restrict__ tw) {
+// One y tile: this thread's column (rows nxs apart from col; ok: it exists)
+// and its neighbours', transformed in place.
+template <int N, bool INV>
+__device__ __forceinline__ void ycols_tile(float2* buf, float2* __restrict__ col, const bool ok, const int nxs,
+                                           const float2* __restrict__ tw) {
   constexpr int TX = ytx<N>();
-  const int tv = min(TX, nxh - kx0);
+  static_assert(kFT % TX == 0, "a thread keeps its column");
   // the first stage reads the columns straight from global memory and the
   // last one writes them back: no staging through shared memory
-  auto load = [&](int t, int y) -> float2 {
-    const float2* src = spec + (plane + y) * nxh + kx0 + t;
-    return t < tv ? (L2LOAD ? __ldcg(src) : *src) : make_float2(0.f, 0.f);
-  };
-  auto store = [&](int t, int y, float2 v) {
-    if (t < tv) spec[(plane + y) * nxh + kx0 + t] = v;
+  auto load = [&](int, int y) -> float2 { return ok ? col[(long long)y * nxs] : make_float2(0.f, 0.f); };
+  auto store = [&](int, int y, float2 v) {
+    if (ok) col[(long long)y * nxs] = v;
   };
   fft_stage0_from<N, TX, kFT, INV>(buf, load);
   fft_ct_range<N, TX, kFT, INV, 1, fft_nstages(N) - 1>(buf, tw);

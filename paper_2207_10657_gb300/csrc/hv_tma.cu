@@ -83,9 +83,9 @@ template <int N> struct TmaLayout {
 }  // namespace
 
 template <int N>
-__device__ __noinline__ void tma_fft_store(float2* buf, float2* spec, const long long nrows, const float2* tw,
+__device__ __noinline__ void tma_fft_store(float2* buf, float2* spec, const long long nrows, const int nxs, const float2* tw,
                                            const long long row0, const long long row_end) {
-  xfwd_fft_store<N, 6>(buf, spec, nrows, tw, row0, row_end);
+  xfwd_fft_store<N, 6>(buf, spec, nrows, nxs, tw, row0, row_end);
 }
 
 // MODE 0: plain (the gradient G : sigma); 1: secant tangent, with this
@@ -96,7 +96,7 @@ template <int N, int MODE>
 __global__ void __launch_bounds__(kFT, kTmaBlocksPerSM)
     kt_xfwd(const __grid_constant__ CUtensorMap tm_in, const __grid_constant__ CUtensorMap tm_dmg,
             const __grid_constant__ CUtensorMap tm_ph, const MatTable<float> mt, float2* __restrict__ spec,
-            const long long nrows, const float2* __restrict__ tw, double* __restrict__ partials, const int ntiles,
+            const long long nrows, const int nxs, const float2* __restrict__ tw, double* __restrict__ partials, const int ntiles,
             int* __restrict__ wait_err, DevScalars* __restrict__ S) {
   using L = TmaLayout<N>;
   constexpr int Q = L::Q, NL = L::NL;
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kFT, kTmaBlocksPerSM)
     // a called (not inlined) transform: inlined into the tile loop, the
     // compiler hoists its loop-invariant index arithmetic out of the loop and
     // holds it in registers across tiles
-    tma_fft_store<N>(buf, spec, nrows, tw, row0, row_end);
+    tma_fft_store<N>(buf, spec, nrows, nxs, tw, row0, row_end);
     __syncthreads();  // the stores have read buf before the next tile's scatter
   }
   if (MODE == 1 && partials) {
@@ -265,10 +265,10 @@ cudaError_t tma_xfwd_n(const GridDesc& g, const float* in, const uint8_t* phase,
     if (dev >= 0 && dev < 64) attr[mi][dev] = 1;
   }
   if (tangent)
-    kt_xfwd<N, 1><<<grid, kFT, smem, st>>>(tin, tdm, tph, mt, spec, g.nrows, tw, partials, ntiles, wait_err,
+    kt_xfwd<N, 1><<<grid, kFT, smem, st>>>(tin, tdm, tph, mt, spec, g.nrows, g.nxs, tw, partials, ntiles, wait_err,
                                            partials ? S : nullptr);
   else
-    kt_xfwd<N, 0><<<grid, kFT, smem, st>>>(tin, tdm, tph, mt, spec, g.nrows, tw, nullptr, ntiles, wait_err, nullptr);
+    kt_xfwd<N, 0><<<grid, kFT, smem, st>>>(tin, tdm, tph, mt, spec, g.nrows, g.nxs, tw, nullptr, ntiles, wait_err, nullptr);
   *nblocks = grid;
   return cudaGetLastError();
 }

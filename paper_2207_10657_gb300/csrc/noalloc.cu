@@ -99,6 +99,7 @@ rve_status rve_project_noalloc(const int dims[3], int ndim, const float* v_dev, 
   g.ny = dims[1];
   g.nz = ndim == 3 ? dims[2] : 1;
   g.nxh = g.nx / 2 + 1;
+  g.nxs = g.nxh;  // unpadded: the scratch array's limit counts Nx/2 + 1 values per row
   g.ncomp = ndim == 3 ? 6 : 3;
   g.nvox = (long long)g.nx * g.ny * g.nz;
   g.nrows = (long long)g.ny * g.nz;

@@ -143,7 +143,7 @@ __device__ __forceinline__ void xfwd_body(const R* __restrict__ in, const uint8_
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
   const long long row0 = (long long)bx * Q;
-  const int npair = (g.ncomp * Q) >> 1, nx = g.nx, nxh = g.nxh, lp = px.lp;
+  const int npair = (g.ncomp * Q) >> 1, nx = g.nx, nxh = g.nxh, nxs = g.nxs, lp = px.lp;
   const XTables tab(buf, g, px, Q, npair, row0, true);
   if (g.nq > 1) xfwd_load<R, MODE, 0>(buf, in, phase, dmg, mt, g, Q, px, row0, ct);
   else if (g.ndim == 3) xfwd_load<R, MODE, 6>(buf, in, phase, dmg, mt, g, Q, px, row0, ct);
@@ -155,8 +155,8 @@ __device__ __forceinline__ void xfwd_body(const R* __restrict__ in, const uint8_
     const C* line = buf + p * lp;
     const C zk = line[tab.at[k]], zm = line[tab.at[k == 0 ? 0 : nx - k]];
     const int ra = tab.row[2 * p], rb = tab.row[2 * p + 1];
-    if (ra >= 0) spec[(long long)ra * nxh + k] = C{(zk.x + zm.x) * (R)0.5, (zk.y - zm.y) * (R)0.5};
-    if (rb >= 0) spec[(long long)rb * nxh + k] = C{(zk.y + zm.y) * (R)0.5, (zm.x - zk.x) * (R)0.5};
+    if (ra >= 0) spec[(long long)ra * nxs + k] = C{(zk.x + zm.x) * (R)0.5, (zk.y - zm.y) * (R)0.5};
+    if (rb >= 0) spec[(long long)rb * nxs + k] = C{(zk.y + zm.y) * (R)0.5, (zm.x - zk.x) * (R)0.5};
   }
 }
 
@@ -177,14 +177,14 @@ __device__ __forceinline__ void ycols_body(Cx<R>* __restrict__ spec, const GridD
   using C = Cx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  const int tx = 1 << ltx, nxh = g.nxh;
+  const int tx = 1 << ltx, nxs = g.nxs;
   // the threads are a multiple of the columns: a thread keeps one column
   int plane, kx;
-  const bool ok = ColTiles(g.ncomp * g.nz, nxh, tx).at(b, threadIdx.x & (tx - 1), &plane, &kx);
-  C* col = spec + (long long)plane * g.ny * nxh + kx;
-  auto load = [=](int, int y, int) -> C { return ok ? col[(long long)y * nxh] : C{0, 0}; };
+  const bool ok = ColTiles(g.ncomp * g.nz, g.nxh, tx).at(b, threadIdx.x & (tx - 1), &plane, &kx);
+  C* col = spec + (long long)plane * g.ny * nxs + kx;
+  auto load = [=](int, int y, int) -> C { return ok ? col[(long long)y * nxs] : C{0, 0}; };
   auto store = [=](int, int y, int, C v) {
-    if (ok) col[(long long)y * nxh] = v;
+    if (ok) col[(long long)y * nxs] = v;
   };
   tile_dit<INV, true, true>(buf, py, TileShape{1, tx, ltx}, tw, load, store);
 }
@@ -213,13 +213,13 @@ __device__ __forceinline__ void zproj_body(Cx<R>* __restrict__ spec, const GridD
   using C = Cx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  const int nz = g.nz, ny = g.ny, nxh = g.nxh, tx = 1 << ltx;
+  const int nz = g.nz, ny = g.ny, nxs = g.nxs, tx = 1 << ltx;
   const int ncl = g.ncomp;  // lines per column: 6, or 36 for Kuhn tetrahedra
   const int t = threadIdx.x & (tx - 1);
   int ky, kx;
-  const bool ok = ColTiles(ny, nxh, tx).at(b, t, &ky, &kx);
-  const long long zs = (long long)ny * nxh;
-  C* col = spec + (long long)ky * nxh + kx;
+  const bool ok = ColTiles(ny, g.nxh, tx).at(b, t, &ky, &kx);
+  const long long zs = (long long)ny * nxs;
+  C* col = spec + (long long)ky * nxs + kx;
   auto load = [=](int c, int z, int) -> C { return ok ? col[(c * nz + z) * zs] : C{0, 0}; };
   auto store = [=](int c, int z, int, C v) {
     if (ok) col[(c * nz + z) * zs] = v;
@@ -301,14 +301,14 @@ __device__ __forceinline__ void yproj2d_body(Cx<R>* __restrict__ spec, const Gri
   using C = Cx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  const int ny = g.ny, nxh = g.nxh, ncl = g.ncomp, tx = 1 << ltx;  // 3 lines per column, or 6 (Kuhn triangles)
+  const int ny = g.ny, nxs = g.nxs, ncl = g.ncomp, tx = 1 << ltx;  // 3 lines per column, or 6 (Kuhn triangles)
   const int t = threadIdx.x & (tx - 1);
   int zero, kx;
-  const bool ok = ColTiles(1, nxh, tx).at(b, t, &zero, &kx);
+  const bool ok = ColTiles(1, g.nxh, tx).at(b, t, &zero, &kx);
   C* col = spec + kx;
-  auto load = [=](int c, int y, int) -> C { return ok ? col[((long long)c * ny + y) * nxh] : C{0, 0}; };
+  auto load = [=](int c, int y, int) -> C { return ok ? col[((long long)c * ny + y) * nxs] : C{0, 0}; };
   auto store = [=](int c, int y, int, C v) {
-    if (ok) col[((long long)c * ny + y) * nxh] = v;
+    if (ok) col[((long long)c * ny + y) * nxs] = v;
   };
   const TileShape ts{ncl, tx, ltx};
   tile_dit<false, true, false>(buf, py, ts, tw, load, NoIo{});
@@ -389,15 +389,15 @@ __device__ __forceinline__ void xinv_body(const Cx<R>* __restrict__ spec, R* __r
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
   __shared__ double red[32];
-  const int nx = g.nx, nxh = g.nxh, half = nx >> 1, lp = px.lp;
+  const int nx = g.nx, nxh = g.nxh, nxs = g.nxs, half = nx >> 1, lp = px.lp;
   const int npair = (g.ncomp * Q) >> 1;
   const XTables tab(buf, g, px, Q, npair, (long long)bx * Q, DOT);
   __syncthreads();
   for (int idx = threadIdx.x; idx < npair * nxh; idx += blockDim.x) {
     const int p = px.dh.div(idx), k = idx - p * nxh;
     const int ra = tab.row[2 * p], rb = tab.row[2 * p + 1];
-    C a = ra >= 0 ? spec[(long long)ra * nxh + k] : C{0, 0};
-    C c = rb >= 0 ? spec[(long long)rb * nxh + k] : C{0, 0};
+    C a = ra >= 0 ? spec[(long long)ra * nxs + k] : C{0, 0};
+    C c = rb >= 0 ? spec[(long long)rb * nxs + k] : C{0, 0};
     if (k == 0 || k == half) a.y = c.y = 0;
     buf[p * lp + px.at_natural(k)] = C{a.x - c.y, a.y + c.x};
     if (k != 0 && k != half) buf[p * lp + px.at_natural(nx - k)] = C{a.x + c.y, c.x - a.y};

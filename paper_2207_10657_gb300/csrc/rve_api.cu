@@ -904,6 +904,7 @@ rve_status rve_create(const int dims[3], int ndim, const uint8_t* phase_ids_dev,
   g.ny = dims[1];
   g.nz = ndim == 3 ? dims[2] : 1;
   g.nxh = g.nx / 2 + 1;
+  g.nxs = spectrum_stride(g.nxh);
   g.ncomp = ndim == 3 ? 6 : 3;
   g.nvox = (long long)g.nx * g.ny * g.nz;
   g.nrows = (long long)g.ny * g.nz;
