@@ -196,6 +196,7 @@ __global__ void __launch_bounds__(kGT, kXYPerSM)
             const DevScalars* __restrict__ S, const MatTable<R> mt, const R* __restrict__ in,
             const uint8_t* __restrict__ phase, const R* __restrict__ dmg, const R* __restrict__ cdp,
             const R* __restrict__ ca, const R* __restrict__ cn, const __grid_constant__ MemberFields ext) {
+  chain_begin();
   __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   ItemQueue items(s_items, wl, BP_X, counter);
@@ -212,6 +213,7 @@ __global__ void __launch_bounds__(kGT, kXYPerSM)
 template <bool YINV>
 __global__ void __launch_bounds__(kGT, kXYPerSM)
     kb_ycols(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter) {
+  chain_begin();
   __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   ItemQueue items(s_items, wl, BP_Y, counter);
@@ -225,6 +227,7 @@ __global__ void __launch_bounds__(kGT, kXYPerSM)
 
 __global__ void __launch_bounds__(kGZ, z_blocks<R>())
     kb_zproj(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter) {
+  chain_begin();
   __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   ItemQueue items(s_items, wl, BP_Z, counter);
@@ -238,6 +241,7 @@ __global__ void __launch_bounds__(kGZ, z_blocks<R>())
 
 __global__ void __launch_bounds__(kGT, kXYPerSM)
     kb_yproj2d(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter) {
+  chain_begin();
   __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   ItemQueue items(s_items, wl, BP_2D, counter);
@@ -254,6 +258,7 @@ __global__ void __launch_bounds__(kGT, kXYPerSM)
     kb_xinv(const BDesc* __restrict__ D, const WLists* __restrict__ wl, int* counter,
             const DevScalars* __restrict__ S, R* __restrict__ out, const R* __restrict__ dotw,
             double* __restrict__ partials, const __grid_constant__ MemberFields ext) {
+  chain_begin();
   __shared__ int s_items[ItemQueue::kItemWords];
   __shared__ __align__(16) int s_desc[sizeof(BDesc) / 4];
   ItemQueue items(s_items, wl, BP_X, counter);
@@ -641,7 +646,7 @@ cudaError_t batch_apply(rve_batch_ctx* c, const R* in, R* out, bool tangent, con
     const bool cons = c->cdp != nullptr;
     const MemberFields none{};
     auto launch = [&](auto kernel) {
-      kernel<<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S, c->mt, in,
+      launch_chained(kernel, grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st, c->dD, c->wl, next_counter(c), c->S, c->mt, in,
                                                                      c->phase, c->D, c->cdp, c->ca, c->cn,
                                                                      ein ? *ein : none);
     };
@@ -657,33 +662,30 @@ cudaError_t batch_apply(rve_batch_ctx* c, const R* in, R* out, bool tangent, con
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (c->any3d) {
-    kb_ycols<false><<<grid_for(c->total[BP_Y], kXYPerSM), kGT, c->smem[BP_Y], c->st>>>(
-        c->dD, c->wl, next_counter(c));
-    kb_zproj<<<grid_for(c->total[BP_Z], z_blocks<R>()), kGZ, c->smem[BP_Z], c->st>>>(c->dD, c->wl, next_counter(c));
-    kb_ycols<true><<<grid_for(c->total[BP_Y], kXYPerSM), kGT, c->smem[BP_Y], c->st>>>(
-        c->dD, c->wl, next_counter(c));
+    launch_chained(kb_ycols<false>, grid_for(c->total[BP_Y], kXYPerSM), kGT, c->smem[BP_Y], c->st, c->dD, c->wl, next_counter(c));
+    launch_chained(kb_zproj, grid_for(c->total[BP_Z], z_blocks<R>()), kGZ, c->smem[BP_Z], c->st, c->dD, c->wl, next_counter(c));
+    launch_chained(kb_ycols<true>, grid_for(c->total[BP_Y], kXYPerSM), kGT, c->smem[BP_Y], c->st, c->dD, c->wl, next_counter(c));
     c->launches += 3;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (c->any2d) {
-    kb_yproj2d<<<grid_for(c->total[BP_2D], kXYPerSM), kGT, c->smem[BP_2D], c->st>>>(
-        c->dD, c->wl, next_counter(c));
+    launch_chained(kb_yproj2d, grid_for(c->total[BP_2D], kXYPerSM), kGT, c->smem[BP_2D], c->st, c->dD, c->wl, next_counter(c));
     ++c->launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const int tot = c->total[BP_X];
   const MemberFields none{};
   if (eout)
-    kb_xinv<0, true><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S,
+    launch_chained(kb_xinv<0, true>, grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st, c->dD, c->wl, next_counter(c), c->S,
                                                                              nullptr, nullptr, nullptr, *eout);
   else if (!dotw)
-    kb_xinv<0, false><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S, out,
+    launch_chained(kb_xinv<0, false>, grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st, c->dD, c->wl, next_counter(c), c->S, out,
                                                                               nullptr, nullptr, none);
   else if (dotw == out)
-    kb_xinv<2, false><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S, out,
+    launch_chained(kb_xinv<2, false>, grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st, c->dD, c->wl, next_counter(c), c->S, out,
                                                                               nullptr, c->part, none);
   else
-    kb_xinv<1, false><<<grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st>>>(c->dD, c->wl, next_counter(c), c->S, out,
+    launch_chained(kb_xinv<1, false>, grid_for(tot, kXYPerSM), kGT, c->smem[BP_X], c->st, c->dD, c->wl, next_counter(c), c->S, out,
                                                                               dotw, c->part, none);
   c->launches += 2;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -8,6 +8,7 @@
 #include "fft_ct.cuh"
 #include "hv_fast.cuh"
 #include "hv_tiles.cuh"
+#include "launch.cuh"
 #include "project.cuh"
 
 namespace rve {
@@ -18,8 +19,9 @@ template <int N, int NC, int MODE>
 __global__ void __launch_bounds__(kFT)
     kf_xfwd(const float* __restrict__ in, const uint8_t* __restrict__ phase, const float* __restrict__ dmg,
             const MatTable<float> mt, float2* __restrict__ spec, const long long nrows, const int nxs, const long long nvox,
-            const float2* __restrict__ tw, double* __restrict__ partials, const float* __restrict__ cdp = nullptr,
-            const float* __restrict__ ca = nullptr, const float* __restrict__ cn = nullptr) {
+            const float2* __restrict__ tw, double* __restrict__ partials, const float* __restrict__ cdp,
+            const float* __restrict__ ca, const float* __restrict__ cn) {
+  chain_begin();
   constexpr int Q = xq<N, NC>();
   __shared__ __align__(16) float2 buf[NC * Q / 2 * N];
   __shared__ double red[32];
@@ -36,10 +38,10 @@ template <int N, int NC, bool DOT, bool CG = false>
 __global__ void __launch_bounds__(kFT, 4)
     kf_xinv(const float2* __restrict__ spec, float* __restrict__ out, const float* __restrict__ dotw,
             double* __restrict__ partials, const long long nrows, const int nxs, const long long nvox,
-            const float2* __restrict__ tw, const float scale, const bool self_dot, float* __restrict__ cz = nullptr,
-            float* __restrict__ cr = nullptr, const float* __restrict__ cd = nullptr,
-            const int* __restrict__ cstatus = nullptr, const double* __restrict__ calpha = nullptr,
-            const double* __restrict__ ctau = nullptr) {
+            const float2* __restrict__ tw, const float scale, const bool self_dot, float* __restrict__ cz,
+            float* __restrict__ cr, const float* __restrict__ cd, const int* __restrict__ cstatus,
+            const double* __restrict__ calpha, const double* __restrict__ ctau) {
+  chain_begin();
   constexpr int Q = xq<N, NC>();
   __shared__ __align__(16) float2 buf[NC * Q / 2 * N];
   __shared__ double red[3 * 32];
@@ -51,6 +53,7 @@ __global__ void __launch_bounds__(kFT, 4)
 template <int N, bool INV>
 __global__ void __launch_bounds__(kFT)
     kf_ycols(float2* __restrict__ spec, const int nxh, const int nxs, const float2* __restrict__ tw) {
+  chain_begin();
   constexpr int TX = ytx<N>();
   __shared__ __align__(16) float2 buf[TX * N];
   const int kx = blockIdx.x * TX + threadIdx.x % TX;
@@ -64,6 +67,7 @@ template <int N> constexpr bool yinplace() { return N == 384; }
 template <int N, bool INV>
 __global__ void __launch_bounds__(kFT)
     kf_ycols_ip(float2* __restrict__ spec, const int nxh, const int nxs, const float2* __restrict__ tw) {
+  chain_begin();
   constexpr int TX = 16;
   __shared__ __align__(16) float2 buf[CtTile<N, TX>::LP * TX];
   const int kx = blockIdx.x * TX + threadIdx.x % TX;
@@ -81,6 +85,7 @@ template <int N>
 __global__ void __launch_bounds__(zthreads<N>(), zminblocks<N>())
     kf_zproj(float2* __restrict__ spec, const int ny, const int nxh, const int nxs, const float2* __restrict__ tw,
              const AxisSyms<float> sy, const unsigned free_mask) {
+  chain_begin();
   constexpr int TX = ztx<N>();
   constexpr int NL = 6 * TX;
   constexpr int NT = zthreads<N>();
@@ -142,6 +147,7 @@ template <int N>
 __global__ void __launch_bounds__(zct_threads<N>(), 2)
     kf_zproj_ip(float2* __restrict__ spec, const int ny, const int nxh, const int nxs, const float2* __restrict__ tw,
              const AxisSyms<float> sy, const unsigned free_mask) {
+  chain_begin();
   constexpr int TX = zct_tx<N>(), NT = zct_threads<N>();
   using T = CtTile<N, TX>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -206,6 +212,7 @@ __global__ void __launch_bounds__(kFT)
     kf_yproj2d(float2* __restrict__ spec, const int nxh, const int nxs, const float2* __restrict__ tw,
                const float2* __restrict__ gdx, const float2* __restrict__ gax, const float2* __restrict__ gdy,
                const float2* __restrict__ gay, const unsigned free_mask) {
+  chain_begin();
   constexpr int TX = p2tx_l<N, NCL>();
   constexpr int NL = NCL * TX;
   __shared__ __align__(16) float2 buf[N * NL];
@@ -265,21 +272,21 @@ static cudaError_t xfwd_n(const GridDesc& g, const float* in, const uint8_t* pha
     const int blocks = (int)((g.nrows + Q - 1) / Q);
     *nblocks = blocks;
     if (tangent && g.nq == 2)
-      kf_xfwd<N, 6, 3><<<blocks, kFT, 0, st>>>(in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd);
+      launch_chained(kf_xfwd<N, 6, 3>, blocks, kFT, 0, st, in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd, nullptr, nullptr, nullptr);
     else if (cons)
-      kf_xfwd<N, 6, 2><<<blocks, kFT, 0, st>>>(in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd, ct->dp, ct->a,
+      launch_chained(kf_xfwd<N, 6, 2>, blocks, kFT, 0, st, in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd, ct->dp, ct->a,
                                                 ct->n);
-    else if (tangent) kf_xfwd<N, 6, 1><<<blocks, kFT, 0, st>>>(in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd);
-    else kf_xfwd<N, 6, 0><<<blocks, kFT, 0, st>>>(in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, nullptr);
+    else if (tangent) launch_chained(kf_xfwd<N, 6, 1>, blocks, kFT, 0, st, in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd, nullptr, nullptr, nullptr);
+    else launch_chained(kf_xfwd<N, 6, 0>, blocks, kFT, 0, st, in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, nullptr, nullptr, nullptr, nullptr);
   } else {
     constexpr int Q = xq<N, 3>();
     const int blocks = (int)((g.nrows + Q - 1) / Q);
     *nblocks = blocks;
     if (cons)
-      kf_xfwd<N, 3, 2><<<blocks, kFT, 0, st>>>(in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd, ct->dp, ct->a,
+      launch_chained(kf_xfwd<N, 3, 2>, blocks, kFT, 0, st, in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd, ct->dp, ct->a,
                                                 ct->n);
-    else if (tangent) kf_xfwd<N, 3, 1><<<blocks, kFT, 0, st>>>(in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd);
-    else kf_xfwd<N, 3, 0><<<blocks, kFT, 0, st>>>(in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, nullptr);
+    else if (tangent) launch_chained(kf_xfwd<N, 3, 1>, blocks, kFT, 0, st, in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, pd, nullptr, nullptr, nullptr);
+    else launch_chained(kf_xfwd<N, 3, 0>, blocks, kFT, 0, st, in, phase, dmg, mt, spec, g.nrows, g.nxs, g.nvox, tw, nullptr, nullptr, nullptr, nullptr);
   }
   return cudaGetLastError();
 }
@@ -292,14 +299,14 @@ static cudaError_t xinv_n(const GridDesc& g, const float2* spec, float* out, con
     constexpr int Q = xq<N, 6>();
     const int blocks = (int)((g.nrows + Q - 1) / Q);
     *nblocks = blocks;
-    if (dot) kf_xinv<N, 6, true><<<blocks, kFT, 0, st>>>(spec, out, dotw, partials, g.nrows, g.nxs, g.nvox, tw, scale, self);
-    else kf_xinv<N, 6, false><<<blocks, kFT, 0, st>>>(spec, out, dotw, partials, g.nrows, g.nxs, g.nvox, tw, scale, self);
+    if (dot) launch_chained(kf_xinv<N, 6, true, false>, blocks, kFT, 0, st, spec, out, dotw, partials, g.nrows, g.nxs, g.nvox, tw, scale, self, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
+    else launch_chained(kf_xinv<N, 6, false, false>, blocks, kFT, 0, st, spec, out, dotw, partials, g.nrows, g.nxs, g.nvox, tw, scale, self, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
   } else {
     constexpr int Q = xq<N, 3>();
     const int blocks = (int)((g.nrows + Q - 1) / Q);
     *nblocks = blocks;
-    if (dot) kf_xinv<N, 3, true><<<blocks, kFT, 0, st>>>(spec, out, dotw, partials, g.nrows, g.nxs, g.nvox, tw, scale, self);
-    else kf_xinv<N, 3, false><<<blocks, kFT, 0, st>>>(spec, out, dotw, partials, g.nrows, g.nxs, g.nvox, tw, scale, self);
+    if (dot) launch_chained(kf_xinv<N, 3, true, false>, blocks, kFT, 0, st, spec, out, dotw, partials, g.nrows, g.nxs, g.nvox, tw, scale, self, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
+    else launch_chained(kf_xinv<N, 3, false, false>, blocks, kFT, 0, st, spec, out, dotw, partials, g.nrows, g.nxs, g.nvox, tw, scale, self, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
   }
   return cudaGetLastError();
 }
@@ -309,12 +316,12 @@ static cudaError_t ycols_n(const GridDesc& g, float2* spec, const float2* tw, bo
   const int planes = g.ncomp * g.nz;
   if constexpr (yinplace<N>()) {
     const dim3 grid((g.nxh + 15) / 16, planes);
-    if (inv) kf_ycols_ip<N, true><<<grid, kFT, 0, st>>>(spec, g.nxh, g.nxs, tw);
-    else kf_ycols_ip<N, false><<<grid, kFT, 0, st>>>(spec, g.nxh, g.nxs, tw);
+    if (inv) launch_chained(kf_ycols_ip<N, true>, grid, kFT, 0, st, spec, g.nxh, g.nxs, tw);
+    else launch_chained(kf_ycols_ip<N, false>, grid, kFT, 0, st, spec, g.nxh, g.nxs, tw);
   } else {
     const dim3 grid((g.nxh + ytx<N>() - 1) / ytx<N>(), planes);
-    if (inv) kf_ycols<N, true><<<grid, kFT, 0, st>>>(spec, g.nxh, g.nxs, tw);
-    else kf_ycols<N, false><<<grid, kFT, 0, st>>>(spec, g.nxh, g.nxs, tw);
+    if (inv) launch_chained(kf_ycols<N, true>, grid, kFT, 0, st, spec, g.nxh, g.nxs, tw);
+    else launch_chained(kf_ycols<N, false>, grid, kFT, 0, st, spec, g.nxh, g.nxs, tw);
   }
   return cudaGetLastError();
 }
@@ -342,7 +349,7 @@ static cudaError_t zproj_n(const GridDesc& g, float2* spec, const SpecWork<float
     if (dev >= 0 && dev < kDevs) attr[dev] = true;
   }
   const AxisSyms<float> sy{{w.gdiff[0], w.gdiff[1], w.gdiff[2]}, {w.gavg[0], w.gavg[1], w.gavg[2]}};
-  kernel<<<dim3((g.nxh + TX - 1) / TX, g.ny), NT, smem, st>>>(spec, g.ny, g.nxh, g.nxs, w.tw[2], sy, w.free_mask);
+  launch_chained(kernel, dim3((g.nxh + TX - 1) / TX, g.ny), NT, smem, st, spec, g.ny, g.nxh, g.nxs, w.tw[2], sy, w.free_mask);
   return cudaGetLastError();
 }
 
@@ -350,11 +357,11 @@ template <int N>
 static cudaError_t yproj2d_n(const GridDesc& g, float2* spec, const SpecWork<float>& w, cudaStream_t st) {
   if (g.ncomp == 6) {
     constexpr int TX = p2tx_l<N, 6>();
-    kf_yproj2d<N, 6><<<(g.nxh + TX - 1) / TX, kFT, 0, st>>>(spec, g.nxh, g.nxs, w.tw[1], w.gdiff[0], w.gavg[0],
+    launch_chained(kf_yproj2d<N, 6>, (g.nxh + TX - 1) / TX, kFT, 0, st, spec, g.nxh, g.nxs, w.tw[1], w.gdiff[0], w.gavg[0],
                                                              w.gdiff[1], w.gavg[1], w.free_mask);
   } else {
     constexpr int TX = p2tx_l<N, 3>();
-    kf_yproj2d<N, 3><<<(g.nxh + TX - 1) / TX, kFT, 0, st>>>(spec, g.nxh, g.nxs, w.tw[1], w.gdiff[0], w.gavg[0],
+    launch_chained(kf_yproj2d<N, 3>, (g.nxh + TX - 1) / TX, kFT, 0, st, spec, g.nxh, g.nxs, w.tw[1], w.gdiff[0], w.gavg[0],
                                                              w.gdiff[1], w.gavg[1], w.free_mask);
   }
   return cudaGetLastError();
@@ -388,13 +395,13 @@ static cudaError_t xinv_cg_n(const GridDesc& g, const float2* spec, float* z, fl
     constexpr int Q = xq<N, 6>();
     const int blocks = (int)((g.nrows + Q - 1) / Q);
     *nblocks = blocks;
-    kf_xinv<N, 6, false, true><<<blocks, kFT, 0, st>>>(spec, nullptr, nullptr, partials, g.nrows, g.nxs, g.nvox, tw, scale,
+    launch_chained(kf_xinv<N, 6, false, true>, blocks, kFT, 0, st, spec, nullptr, nullptr, partials, g.nrows, g.nxs, g.nvox, tw, scale,
                                                        false, z, r, d, status, alpha, tau);
   } else {
     constexpr int Q = xq<N, 3>();
     const int blocks = (int)((g.nrows + Q - 1) / Q);
     *nblocks = blocks;
-    kf_xinv<N, 3, false, true><<<blocks, kFT, 0, st>>>(spec, nullptr, nullptr, partials, g.nrows, g.nxs, g.nvox, tw, scale,
+    launch_chained(kf_xinv<N, 3, false, true>, blocks, kFT, 0, st, spec, nullptr, nullptr, partials, g.nrows, g.nxs, g.nvox, tw, scale,
                                                        false, z, r, d, status, alpha, tau);
   }
   return cudaGetLastError();

@@ -269,9 +269,9 @@ static cudaError_t spectral_middle(const GridDesc& g, SpecWork<R>& w, cudaStream
         if (!w.generic && pass == 1 && fast_size(g.nz)) e = fast_zproj(g, w.spec, w, st);
       }
       if (e == cudaErrorNotSupported) {
-        if (pass == 0) k_ycols<R, false><<<gt.yblocks, kGT, gt.ysmem, st>>>(w.spec, g, w.lty, w.py, w.tw[1]);
-        else if (pass == 2) k_ycols<R, true><<<gt.yblocks, kGT, gt.ysmem, st>>>(w.spec, g, w.lty, w.py, w.tw[1]);
-        else k_zproj<R><<<gt.zblocks, kGZ, gt.zsmem, st>>>(w.spec, g, w.ltz, w.pz, w.tw[2], sy, w.free_mask);
+        if (pass == 0) launch_chained(k_ycols<R, false>, gt.yblocks, kGT, gt.ysmem, st, w.spec, g, w.lty, w.py, w.tw[1]);
+        else if (pass == 2) launch_chained(k_ycols<R, true>, gt.yblocks, kGT, gt.ysmem, st, w.spec, g, w.lty, w.py, w.tw[1]);
+        else launch_chained(k_zproj<R>, gt.zblocks, kGZ, gt.zsmem, st, w.spec, g, w.ltz, w.pz, w.tw[2], sy, w.free_mask);
         e = cudaGetLastError();
       }
       if (e != cudaSuccess) return e;
@@ -284,7 +284,7 @@ static cudaError_t spectral_middle(const GridDesc& g, SpecWork<R>& w, cudaStream
       if (!w.generic && fast_size(g.ny)) e = fast_yproj2d(g, w.spec, w, st);
     }
     if (e == cudaErrorNotSupported) {
-      k_yproj2d<R><<<gt.zblocks, kGT, gt.zsmem, st>>>(w.spec, g, w.ltz, w.py, w.tw[1], sy, w.free_mask);
+      launch_chained(k_yproj2d<R>, gt.zblocks, kGT, gt.zsmem, st, w.spec, g, w.ltz, w.py, w.tw[1], sy, w.free_mask);
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
@@ -345,11 +345,11 @@ cudaError_t spectral_apply(const GridDesc& g, SpecWork<R>& w, const MatTable<R>&
   }
   if (e == cudaErrorNotSupported) {
     if (mode == XIn::Tangent && w.cons.dp)
-      k_xfwd<R, 2><<<xblocks, kGT, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0], w.cons);
+      launch_chained(k_xfwd<R, 2>, xblocks, kGT, xsm, st, in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0], w.cons);
     else if (mode == XIn::Tangent)
-      k_xfwd<R, 1><<<xblocks, kGT, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0], w.cons);
+      launch_chained(k_xfwd<R, 1>, xblocks, kGT, xsm, st, in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0], w.cons);
     else
-      k_xfwd<R, 0><<<xblocks, kGT, xsm, st>>>(in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0],
+      launch_chained(k_xfwd<R, 0>, xblocks, kGT, xsm, st, in, phase, damage, mt, w.spec, g, w.qx, w.px, w.tw[0],
                                                     ConsTan<R>{});
     e = cudaGetLastError();
   }
@@ -375,10 +375,10 @@ cudaError_t spectral_apply(const GridDesc& g, SpecWork<R>& w, const MatTable<R>&
   if (e == cudaErrorNotSupported) {
     nblocks = xblocks;
     if (dot)
-      k_xinv<R, true><<<xblocks, kGT, xsm, st>>>(w.spec, out, self ? nullptr : dot_with, w.partials, g, w.qx,
+      launch_chained(k_xinv<R, true>, xblocks, kGT, xsm, st, w.spec, out, self ? nullptr : dot_with, w.partials, g, w.qx,
                                                        w.px, w.tw[0], scale, self);
     else
-      k_xinv<R, false><<<xblocks, kGT, xsm, st>>>(w.spec, out, nullptr, nullptr, g, w.qx, w.px, w.tw[0],
+      launch_chained(k_xinv<R, false>, xblocks, kGT, xsm, st, w.spec, out, nullptr, nullptr, g, w.qx, w.px, w.tw[0],
                                                         scale, false);
     e = cudaGetLastError();
   }

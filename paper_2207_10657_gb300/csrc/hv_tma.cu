@@ -22,6 +22,7 @@
 
 #include "hv_tiles.cuh"
 #include "hv_tma.cuh"
+#include "launch.cuh"
 #include "scalar_logic.cuh"
 
 namespace rve {
@@ -98,6 +99,7 @@ __global__ void __launch_bounds__(kFT, kTmaBlocksPerSM)
             const __grid_constant__ CUtensorMap tm_ph, const MatTable<float> mt, float2* __restrict__ spec,
             const long long nrows, const int nxs, const float2* __restrict__ tw, double* __restrict__ partials, const int ntiles,
             int* __restrict__ wait_err, DevScalars* __restrict__ S) {
+  chain_begin();
   using L = TmaLayout<N>;
   constexpr int Q = L::Q, NL = L::NL;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -265,10 +267,10 @@ cudaError_t tma_xfwd_n(const GridDesc& g, const float* in, const uint8_t* phase,
     if (dev >= 0 && dev < 64) attr[mi][dev] = 1;
   }
   if (tangent)
-    kt_xfwd<N, 1><<<grid, kFT, smem, st>>>(tin, tdm, tph, mt, spec, g.nrows, g.nxs, tw, partials, ntiles, wait_err,
+    launch_chained(kt_xfwd<N, 1>, grid, kFT, smem, st, tin, tdm, tph, mt, spec, g.nrows, g.nxs, tw, partials, ntiles, wait_err,
                                            partials ? S : nullptr);
   else
-    kt_xfwd<N, 0><<<grid, kFT, smem, st>>>(tin, tdm, tph, mt, spec, g.nrows, g.nxs, tw, nullptr, ntiles, wait_err, nullptr);
+    launch_chained(kt_xfwd<N, 0>, grid, kFT, smem, st, tin, tdm, tph, mt, spec, g.nrows, g.nxs, tw, nullptr, ntiles, wait_err, nullptr);
   *nblocks = grid;
   return cudaGetLastError();
 }

@@ -5,6 +5,7 @@
 
 #include "fft_inplace.cuh"
 #include "hv_passes.cuh"
+#include "launch.cuh"
 #include "project.cuh"
 
 namespace rve {
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(kGT, xy_blocks<R>())
     k_xfwd(const R* __restrict__ in, const uint8_t* __restrict__ phase, const R* __restrict__ dmg,
            const MatTable<R> mt, Cx<R>* __restrict__ spec, const GridDesc g, const int Q,
            const __grid_constant__ AxisPlan px, const Cx<R>* __restrict__ tw, const ConsTan<R> ct) {
+  chain_begin();
   xfwd_body<R, MODE>(in, phase, dmg, mt, spec, g, Q, px, tw, blockIdx.x, ct);
 }
 
@@ -193,6 +195,7 @@ template <typename R, bool INV>
 __global__ void __launch_bounds__(kGT, xy_blocks<R>())
     k_ycols(Cx<R>* __restrict__ spec, const GridDesc g, const int ltx, const __grid_constant__ AxisPlan py,
             const Cx<R>* __restrict__ tw) {
+  chain_begin();
   ycols_body<R, INV>(spec, g, ltx, py, tw, blockIdx.x);
 }
 
@@ -290,6 +293,7 @@ template <typename R>
 __global__ void __launch_bounds__(kGZ, z_blocks<R>())
     k_zproj(Cx<R>* __restrict__ spec, const GridDesc g, const int ltx, const __grid_constant__ AxisPlan pz,
             const Cx<R>* __restrict__ tw, const AxisSyms<R> sy, const unsigned free_mask) {
+  chain_begin();
   zproj_body<R>(spec, g, ltx, pz, tw, sy, free_mask, blockIdx.x);
 }
 
@@ -371,6 +375,7 @@ template <typename R>
 __global__ void __launch_bounds__(kGT, xy_blocks<R>())
     k_yproj2d(Cx<R>* __restrict__ spec, const GridDesc g, const int ltx, const __grid_constant__ AxisPlan py,
               const Cx<R>* __restrict__ tw, const AxisSyms<R> sy, const unsigned free_mask) {
+  chain_begin();
   yproj2d_body<R>(spec, g, ltx, py, tw, sy, free_mask, blockIdx.x);
 }
 
@@ -439,6 +444,7 @@ __global__ void __launch_bounds__(kGT, xy_blocks<R>())
     k_xinv(const Cx<R>* __restrict__ spec, R* __restrict__ out, const R* __restrict__ dotw,
            double* __restrict__ partials, const GridDesc g, const int Q, const __grid_constant__ AxisPlan px,
            const Cx<R>* __restrict__ tw, const R scale, const bool self_dot) {
+  chain_begin();
   xinv_body<R, DOT>(spec, out, dotw, DOT ? partials + blockIdx.x : nullptr, g, Q, px, tw, scale, self_dot,
                     blockIdx.x);
 }
