@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(kFT)
             const float* __restrict__ ca, const float* __restrict__ cn) {
   chain_begin();
   constexpr int Q = xq<N, NC>();
-  __shared__ __align__(16) float2 buf[NC * Q / 2 * N];
+  __shared__ __align__(16) float2 buf[xlines<N, NC * Q / 2>()];
   __shared__ double red[32];
   const long long row0 = (long long)blockIdx.x * Q;
   const float acc = xfwd_rows<N, NC, MODE>(buf, in, phase, dmg, mt, spec, nrows, nxs, nvox, tw, row0, nrows, cdp, ca, cn);
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kFT)
 }
 
 // The in-place form, for the length whose Stockham tile takes ten columns (80
-// of the 128 bytes of a segment): 16 columns, 606 -> 540 us per pass at 384^3.
+// of the 128 bytes of a segment): 16 columns, 606 -> 471 us per pass at 384^3.
 template <int N> constexpr bool yinplace() { return N == 384; }
 
 template <int N, bool INV>
@@ -136,12 +136,13 @@ __global__ void __launch_bounds__(zthreads<N>(), zminblocks<N>())
 
 // The in-place form (fft_ct.cuh), for the length whose Stockham tile (72
 // butterfly values a thread) had to be staged through shared memory: 2141 ->
-// 1412 us per pass at 384^3.  The powers of two and 192 stay on the Stockham
+// 1357 us per pass at 384^3.  The powers of two and 192 stay on the Stockham
 // form, which needs no reordering between the projection and the inverse
 // (256^3: 321 us against 391 us in place).
 template <int N> constexpr bool zinplace() { return N == 384; }
-template <int N> constexpr int zct_tx() { return 4; }       // 75 KB: two blocks per SM
-template <int N> constexpr int zct_threads() { return 512; }
+template <int N> constexpr int zct_tx() { return 4; }  // 75 KB: two blocks per SM
+// 256 threads at 128 registers 4241 us per 384^3 product, 512 at 64 registers 4291 us
+template <int N> constexpr int zct_threads() { return 256; }
 
 template <int N>
 __global__ void __launch_bounds__(zct_threads<N>(), 2)

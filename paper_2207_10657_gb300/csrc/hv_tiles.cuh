@@ -4,7 +4,7 @@
 // 384.
 #pragma once
 
-#include "fft_fast.cuh"
+#include "fft_ct.cuh"
 #include "hv_passes.cuh"
 
 namespace rve {
@@ -52,6 +52,38 @@ template <int N, int NROW> struct RowItems {
   __device__ __forceinline__ static bool valid(int rho, int) { return rho < NROW; }
 };
 
+
+// ------------------------------------------------------------ x lines
+// Forward transform of NL interleaved lines of an x tile.  At 384 points (8 x
+// 4 x 4 x 3) in place (fft_ct.cuh, three stages with one barrier each: 949 ->
+// 856 us per pass at 384^3), at the other lengths self-sorting: element x of
+// the input and frequency k of the output sit at rows xin<N>(x) and xout<N>(k)
+// of the tile.  The x-inverse, whose rows leave in natural order, stays
+// self-sorting at 384 too (975 us; in place 1177 us).
+template <int N> constexpr bool xinplace() { return N == 384; }
+template <int N, int NL> constexpr int xlines() {
+  if constexpr (xinplace<N>()) return CtTile<N, NL>::LP * NL;
+  else return N * NL;
+}
+template <int N, int NL> __device__ __forceinline__ int xin(int x) {
+  if constexpr (xinplace<N>()) return CtTile<N, NL>::natural(x);
+  else return x;
+}
+template <int N, int NL> __device__ __forceinline__ int xout(int k) {
+  if constexpr (xinplace<N>()) return CtTile<N, NL>::freq(k);
+  else return k;
+}
+struct NoStage {
+  template <typename... A> __device__ __forceinline__ int operator()(A...) const { return 0; }
+};
+template <int N, int NL> __device__ __forceinline__ void xfft(float2* buf, const float2* __restrict__ tw) {
+  if constexpr (xinplace<N>()) {
+    ct_dit<N, NL, 1, kFT, false, false, false>(buf, tw, NoStage{}, NoStage{});
+    __syncthreads();
+  } else {
+    fft_ct<N, NL, kFT, false>(buf, tw);
+  }
+}
 
 // ------------------------------------------------------------ x forward
 template <int N, int NC>
@@ -151,7 +183,7 @@ __device__ __forceinline__ float xfwd_rows(float2* buf, const float* __restrict_
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           const int rho = q * NC + c;
-          reinterpret_cast<float*>(&buf[x * NL + (rho >> 1)])[rho & 1] = v[b][c];
+          reinterpret_cast<float*>(&buf[xin<N, NL>(x) * NL + (rho >> 1)])[rho & 1] = v[b][c];
         }
       }
     }
@@ -175,18 +207,18 @@ __device__ __forceinline__ void xfwd_fft_store(float2* buf, float2* __restrict__
                                                const long long row_end) {
   constexpr int Q = xq<N, NC>();
   constexpr int NL = NC * Q / 2;
-  fft_ct<N, NL, kFT, false>(buf, tw);
+  xfft<N, NL>(buf, tw);
   constexpr int KB = N / 2, GB = kFT / KB, JB = (NL + GB - 1) / GB;
   const long long plane = nrows * nxs;
   {
     const int g = threadIdx.x / KB, k = threadIdx.x - (threadIdx.x / KB) * KB;
-    const int km = k == 0 ? 0 : N - k;
+    const int ak = xout<N, NL>(k), am = xout<N, NL>(k == 0 ? 0 : N - k);
     if (g < GB) {
 #pragma unroll
       for (int j = 0; j < JB; ++j) {
         const int p = g + j * GB;
         if (JB * GB == NL || p < NL) {
-          const float2 zk = buf[k * NL + p], zm = buf[km * NL + p];
+          const float2 zk = buf[ak * NL + p], zm = buf[am * NL + p];
           const float2 xa = make_float2((zk.x + zm.x) * 0.5f, (zk.y - zm.y) * 0.5f);
           const float2 xb = make_float2((zk.y + zm.y) * 0.5f, (zm.x - zk.x) * 0.5f);
 #pragma unroll
@@ -200,7 +232,7 @@ __device__ __forceinline__ void xfwd_fft_store(float2* buf, float2* __restrict__
     }
     if (threadIdx.x < NL) {
       const int p = threadIdx.x;
-      const float2 z = buf[KB * NL + p];
+      const float2 z = buf[xout<N, NL>(KB) * NL + p];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int rho = 2 * p + h;
