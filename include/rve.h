@@ -376,7 +376,9 @@ rve_status rve_batch_create(int n, const int* dims_host, const int* ndims_host,
 rve_status rve_batch_solve_step(rve_batch_t, const double* dE_host, const uint8_t* free_mask_host,
                                 rve_step_report* reps_host);
 /* One batched Hessian-vector product out_i = G:((1-D_i)C:v_i) on every
- * member (host arrays of n device pointers, ncomp*Nvox_i floats each). */
+ * member (host arrays of n device pointers, ncomp*Nvox_i floats each; the
+ * fields may alias: every input is read before any output is written).
+ * RVE_ERR_ARG on a NULL pointer. */
 rve_status rve_batch_hessp(rve_batch_t, const float* const* v_dev, float* const* out_dev);
 /* Frozen damage of member i (Nvox_i floats), as rve_set_damage. */
 rve_status rve_batch_set_damage(rve_batch_t, int i, const float* damage_dev);

@@ -47,3 +47,35 @@ def test_product_matches_oracle(dims, precision):
     rve = oracle.RVE(pm, [oracle.Phase(1.0, 0.3, True, 1e-4, 1e-3), oracle.Phase(10.0, 0.2)])
     ref = rve.hessp(Dt.double().cpu().numpy(), vt.double().cpu().numpy())
     assert np.linalg.norm(got - ref) <= TOL[precision] * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n", [1, 33, 256])
+def test_batched_product_in_place_of_many_members(n):
+    """Work lists of one, of a little more than a warp's and of the largest
+    number of members; the products overwrite their inputs."""
+    from paper_2207_10657_gb300 import Phase, RVEBatch, RVESolver, build
+    from paper_2207_10657_gb300 import binding as B
+    build.build()
+    phases = [Phase(1.0, 0.3, True, 1e-4, 1e-3), Phase(10.0, 0.2)]
+    kinds = [(8, 6), (10, 4, 6), (12, 18)]
+    dims = [kinds[i % 3] for i in range(n)]
+    pms = [_cell(d, i) for i, d in enumerate(dims)]
+    Ds = [torch.from_numpy(damage_snapshot(pm, dmax=0.9, seed=i)).float().cuda() for i, pm in enumerate(pms)]
+    vs = [torch.from_numpy(random_field(6 if len(d) == 3 else 3, d, seed=i)).float().cuda()
+          for i, d in enumerate(dims)]
+    ref = []
+    for d, pm, D, v in zip(dims, pms, Ds, vs):
+        s = RVESolver(d, pm, phases, passes=1)
+        s.set_damage(D)
+        ref.append(s.hessp(v))
+        s.close()
+    b = RVEBatch(dims, pms, phases)
+    for i, D in enumerate(Ds):
+        b.set_damage(i, D)
+    B.rve_batch_hessp(b.h, [v.data_ptr() for v in vs], [v.data_ptr() for v in vs])
+    torch.cuda.synchronize()
+    for got, want in zip(vs, ref):
+        assert float((got - want).norm()) <= TOL[32] * float(want.norm())
+    with pytest.raises(B.RveError):
+        B.rve_batch_hessp(b.h, [0] * n, [v.data_ptr() for v in vs])
+    b.close()
