@@ -63,8 +63,9 @@ void finish_plan(AxisPlan& p) {
 }
 
 // The radix sequence of the compiled passes (8s, 4s, 2, 3s, 5s), successive
-// factors below 8 joined in pairs so that the fewest stages result.
-static void make_plan(int n, AxisPlan& p, bool keep) {
+// factors below 8 joined in pairs so that the fewest stages result; `narrow`:
+// 4s in place of the 8s and no pairs (kNarrowMax).
+static void make_plan(int n, AxisPlan& p, bool keep, bool narrow) {
   p = AxisPlan{};
   p.n = n;
   p.keep_order = keep ? 1 : 0;
@@ -76,12 +77,17 @@ static void make_plan(int n, AxisPlan& p, bool keep) {
   else if (rem == 1) {
     if (n8 > 0) { --n8; n4 = 2; } else n2 = 1;
   }
+  if (narrow) {
+    n8 = 0;
+    n4 = twos / 2;
+    n2 = twos % 2;
+  }
   for (int i = 0; i < n8; ++i) f[nf++] = 8;
   for (int i = 0; i < n4; ++i) f[nf++] = 4;
   for (int i = 0; i < n2; ++i) f[nf++] = 2;
   while (m % 3 == 0) { m /= 3; f[nf++] = 3; }
   while (m % 5 == 0) { m /= 5; f[nf++] = 5; }
-  auto pairs = [&](int i) { return i >= 0 && i + 1 < nf && f[i] < 8 && f[i] * f[i + 1] <= 20; };
+  auto pairs = [&](int i) { return !narrow && i >= 0 && i + 1 < nf && f[i] < 8 && f[i] * f[i + 1] <= 20; };
   // from the back, and from the front: keep the shorter, then the one with
   // the smaller largest radix
   int best[16], nb = 99, mx = 99;
@@ -159,6 +165,16 @@ GenericTiles<R>::GenericTiles(const GridDesc& g, int qx, int lty, int ltz, const
 template struct GenericTiles<float>;
 template struct GenericTiles<double>;
 
+// FP64 cells of up to this many field values take radices 2, 3, 4 and 5 only.
+// Such a grid leaves most SMs a warp or two, and an FP64 instruction occupies
+// its scheduler for 64 cycles however few lanes it has: a stage's time is the
+// number of instructions of ONE butterfly, so small butterflies spread over
+// more warps win.  Products, wide -> narrow: 16^2 33.7 -> 22.1 us, 60x90 46.5 ->
+// 38.4, 128^2 (49152 values) 53.8 -> 37.7, 16^3 51.8 -> 35.3; past the line
+// the pipe is full and the extra trips through shared memory lose: 256^2 and
+// 32^3 (196608 values) 52.3 -> 62.6 and 62.3 -> 67.3.
+constexpr long long kNarrowMax = 65536;
+
 // Plans and tiles.  A tile is as large as keeps its threads busy (about one
 // butterfly each, 128-byte column segments) and as small as leaves every SM
 // work: with one tile size for all grids, each pass of a 32^2 cell ran on ONE
@@ -169,9 +185,10 @@ cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w) {
   using C = Cx<R>;
   // FP32 cells of one element per voxel keep their roundings (zproj_body)
   const bool keep = std::is_same<R, float>::value && g.nq == 1;
-  make_plan(g.nx, w.px, keep);
-  make_plan(g.ny, w.py, keep);
-  make_plan(g.ndim == 3 ? g.nz : 1, w.pz, keep);
+  const bool narrow = std::is_same<R, double>::value && g.nvox * g.ncomp <= kNarrowMax;
+  make_plan(g.nx, w.px, keep, narrow);
+  make_plan(g.ny, w.py, keep, narrow);
+  make_plan(g.ndim == 3 ? g.nz : 1, w.pz, keep, narrow);
   w.px.dc = FastDiv::by(g.ncomp);
   const int wave = 2 * 152;              // blocks that give every SM two
   const int q1 = (g.ncomp & 1) ? 2 : 1;  // rows come in pairs where ncomp is odd
