@@ -33,6 +33,15 @@ constexpr int kMaxBatch = 256;
 // latency, so two more blocks than the single-grid kernels pay here (96 cells
 // 2.87 -> 2.70 ms; a single 160x120x90 grid 199 -> 206 us)
 constexpr int kXYPerSM = 8;
+// Items that a batched launch should have at least, shared out over the
+// members of one dimension by their field values: a member's tiles shrink only
+// as far as its share asks.  With the rule of a grid alone (kWave each) 256
+// cells of 16^3 had 65536 x items of three lines each, and an item's start
+// outweighed its work: load step of 256 cells of 16^3 51.9 -> 15.6 ms, of 64
+// cells of 24^3 27.3 -> 11.0 ms, product of 96 cells of 32^3 1247 -> 454 us, of 96
+// uneven cells 2398 -> 2215 us (8 cells of 512^2 145 -> 148 us).  8 x 152: 8
+// cells of 16^3 53 -> 66 us, large members alike.
+constexpr int kBatchWave = kWave;
 constexpr long long kVecChunk = 16384;  // field elements per vector item (multiple of 4)
 constexpr long long kVoxChunk = 4096;   // voxels per constitutive item (multiple of 4)
 
@@ -1028,6 +1037,7 @@ rve_status batch_init(rve_batch_ctx* c, const int* dims, const int* ndims, const
   c->desc.resize(n);
   c->radius_set.assign(n, 0);
   for (int p = 0; p < BP_N; ++p) c->hstart[p].assign(n + 1, 0);
+  double field_values[4] = {0, 0, 0, 0};  // of the members of each dimension
   for (int i = 0; i < n; ++i) {
     GridDesc& g = c->g[i];
     g.ndim = ndims[i];
@@ -1041,7 +1051,12 @@ rve_status batch_init(rve_batch_ctx* c, const int* dims, const int* ndims, const
     g.nrows = (long long)g.ny * g.nz;
     if (g.ndim == 3) c->any3d = true;
     else c->any2d = true;
-    BCK(spectral_setup<R>(g, c->sw[i]), "spectral setup");
+    field_values[g.ndim] += (double)(g.ncomp * g.nvox);
+  }
+  for (int i = 0; i < n; ++i) {
+    const GridDesc& g = c->g[i];
+    const int share = (int)std::ceil(kBatchWave * ((double)(g.ncomp * g.nvox) / field_values[g.ndim]));
+    BCK(spectral_setup<R>(g, c->sw[i], share), "spectral setup");
     const SpecWork<R>& w = c->sw[i];
     BDesc& d = c->desc[i];
     d.g = g;
@@ -1145,8 +1160,8 @@ rve_status batch_init(rve_batch_ctx* c, const int* dims, const int* ndims, const
 // ---------------------------------------------------------------- autotune
 // A schedule of the batched spectral passes: every member's x / y / z tile
 // (rows per x item, kx columns per y item and per z item) divided by
-// sx / sy / sz (the tiles of spectral_setup are the largest the per-thread
-// element budgets allow, so only smaller ones are candidates), and the
+// sx / sy / sz (plan_tiles takes the largest that its budgets and the member's
+// share of the launch allow, so only smaller ones are candidates), and the
 // radix order of every axis plan natural or reversed (any order is a valid
 // factorisation).  Work-item counts, dynamic shared memory, the
 // partial-sum buffer and the device descriptors follow; captured graphs are

@@ -176,12 +176,12 @@ template struct GenericTiles<double>;
 constexpr long long kNarrowMax = 65536;
 
 // Plans and tiles.  A tile is as large as keeps its threads busy (about one
-// butterfly each, 128-byte column segments) and as small as leaves every SM
-// work: with one tile size for all grids, each pass of a 32^2 cell ran on ONE
+// butterfly each, 128-byte column segments) and as small as gives the grid
+// `wave` blocks, which alone on the chip leaves every SM work: with one tile size for all grids, each pass of a 32^2 cell ran on ONE
 // SM (FP64 product 129 -> 35 us with 16-17 blocks per pass).  Columns do not
 // go below the 32 bytes of a memory sector while a tile fits a block.
 template <typename R>
-cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w) {
+void plan_tiles(const GridDesc& g, SpecWork<R>& w, int wave) {
   using C = Cx<R>;
   // FP32 cells of one element per voxel keep their roundings (zproj_body)
   const bool keep = std::is_same<R, float>::value && g.nq == 1;
@@ -190,7 +190,6 @@ cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w) {
   make_plan(g.ny, w.py, keep, narrow);
   make_plan(g.ndim == 3 ? g.nz : 1, w.pz, keep, narrow);
   w.px.dc = FastDiv::by(g.ncomp);
-  const int wave = 2 * 152;              // blocks that give every SM two
   const int q1 = (g.ncomp & 1) ? 2 : 1;  // rows come in pairs where ncomp is odd
   // x: about 2048 elements (16 KB in FP32) per block
   long long q = std::max<long long>(q1, 2 * 2048 / ((long long)g.ncomp * g.nx));
@@ -209,6 +208,11 @@ cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w) {
   w.lty = g.ndim == 3 ? columns(w.py, 1, g.ncomp * g.nz, 4096, 1 << 30) : 0;
   if (g.ndim == 3) w.ltz = columns(w.pz, g.ncomp, g.ny, sizeof(C) == 8 ? 6144 : 3072, kHold * kGZ);
   else w.ltz = columns(w.py, g.ncomp, 1, 3072, kHold2 * kGT);
+}
+
+template <typename R>
+cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w, int wave) {
+  plan_tiles<R>(g, w, wave);
   // opt in to large dynamic shared memory
   cudaFuncSetAttribute(k_xfwd<R, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
   cudaFuncSetAttribute(k_xfwd<R, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
@@ -223,9 +227,9 @@ cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w) {
 }
 
 template <typename R>
-cudaError_t spectral_setup(const GridDesc& g, SpecWork<R>& w) {
+cudaError_t spectral_setup(const GridDesc& g, SpecWork<R>& w, int wave) {
   using C = Cx<R>;
-  cudaError_t e = spectral_plan<R>(g, w);
+  cudaError_t e = spectral_plan<R>(g, w, wave);
   if (e != cudaSuccess) return e;
   const int ns[3] = {g.nx, g.ny, g.nz};
   for (int a = 0; a < g.ndim; ++a)
@@ -473,9 +477,11 @@ cudaError_t spectral_hv_cg(const GridDesc& g, SpecWork<float>& w, const MatTable
   return cudaSuccess;
 }
 
-template cudaError_t spectral_setup<float>(const GridDesc&, SpecWork<float>&);
-template cudaError_t spectral_setup<double>(const GridDesc&, SpecWork<double>&);
-template cudaError_t spectral_plan<float>(const GridDesc&, SpecWork<float>&);
+template cudaError_t spectral_setup<float>(const GridDesc&, SpecWork<float>&, int);
+template cudaError_t spectral_setup<double>(const GridDesc&, SpecWork<double>&, int);
+template cudaError_t spectral_plan<float>(const GridDesc&, SpecWork<float>&, int);
+template void plan_tiles<float>(const GridDesc&, SpecWork<float>&, int);
+template void plan_tiles<double>(const GridDesc&, SpecWork<double>&, int);
 template void spectral_free<float>(SpecWork<float>&);
 template void spectral_free<double>(SpecWork<double>&);
 template cudaError_t spectral_apply<float>(const GridDesc&, SpecWork<float>&, const MatTable<float>&, const float*,

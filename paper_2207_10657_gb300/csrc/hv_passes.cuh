@@ -85,14 +85,22 @@ cudaError_t spectral_hv_cg(const GridDesc& g, SpecWork<float>& w, const MatTable
                            const uint8_t* phase, const float* damage, float* z, float* r, DevScalars* S,
                            cudaStream_t st, long long* nlaunch);
 
+constexpr int kWave = 2 * 152;  // blocks that give every SM two
+
+// wave: blocks that this grid's generic passes should have at least, where
+// its size allows (kWave: the grid has a launch to itself; a member of a
+// batch: its share of the batch's launches).
 template <typename R>
-cudaError_t spectral_setup(const GridDesc& g, SpecWork<R>& w);
+cudaError_t spectral_setup(const GridDesc& g, SpecWork<R>& w, int wave = kWave);
 template <typename R>
 void spectral_free(SpecWork<R>& w);
-// Plans and tile sizes only, no device allocation (the caller provides
-// the tables and the spectrum storage in SpecWork).
+// Plans and tile sizes of the generic passes; host work only.
 template <typename R>
-cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w);
+void plan_tiles(const GridDesc& g, SpecWork<R>& w, int wave = kWave);
+// plan_tiles and the kernels' shared-memory attributes, no device allocation
+// (the caller provides the tables and the spectrum storage in SpecWork).
+template <typename R>
+cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w, int wave = kWave);
 // Tile sizes and the blocks / dynamic shared memory they give, for the
 // generic passes with these plans.
 template <typename R> struct GenericTiles {
