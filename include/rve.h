@@ -377,8 +377,10 @@ rve_status rve_batch_solve_step(rve_batch_t, const double* dE_host, const uint8_
                                 rve_step_report* reps_host);
 /* One batched Hessian-vector product out_i = G:((1-D_i)C:v_i) on every
  * member (host arrays of n device pointers, ncomp*Nvox_i floats each; the
- * fields may alias: every input is read before any output is written).
- * RVE_ERR_ARG on a NULL pointer. */
+ * fields may alias: every input is read before any output is written, and
+ * outputs that share memory are written in member order).  RVE_ERR_ARG on a
+ * NULL pointer.  Fields in memory of the current device, aligned to floats,
+ * are used in place; others are copied. */
 rve_status rve_batch_hessp(rve_batch_t, const float* const* v_dev, float* const* out_dev);
 /* Frozen damage of member i (Nvox_i floats), as rve_set_damage. */
 rve_status rve_batch_set_damage(rve_batch_t, int i, const float* damage_dev);

@@ -12,8 +12,10 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <cstdint>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/rve.h"
@@ -1247,6 +1249,35 @@ rve_status time_products(rve_batch_ctx* c, int reps, double* ms) {
   return RVE_OK;
 }
 
+// A member field that the kernels can read and write where it is: memory of
+// this device (or managed), aligned to its elements.  Any other pointer goes
+// through a copy, which takes what cudaMemcpyAsync takes (another device's
+// memory, bytes at any address) and returns an error for the rest, where a
+// kernel would fault.
+bool kernels_reach(const void* p, int dev) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const bool here = (a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged;
+  return here && reinterpret_cast<uintptr_t>(p) % alignof(R) == 0;
+}
+
+// Two outputs share memory (one scratch field for members whose products are
+// not wanted): the kernels would write it in no order, copies in member order.
+bool outputs_overlap(const rve_batch_ctx* c, float* const* out) {
+  std::vector<std::pair<uintptr_t, uintptr_t>> r(c->n);
+  for (int i = 0; i < c->n; ++i) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(out[i]);
+    r[i] = {a, a + (uintptr_t)(c->g[i].ncomp * c->g[i].nvox) * sizeof(R)};
+  }
+  std::sort(r.begin(), r.end());
+  for (int i = 1; i < c->n; ++i)
+    if (r[i].first < r[i - 1].second) return true;
+  return false;
+}
+
 }  // namespace
 
 // ================================================================ C ABI
@@ -1320,11 +1351,21 @@ rve_status rve_batch_solve_step(rve_batch_t c, const double* dE, const uint8_t* 
 rve_status rve_batch_hessp(rve_batch_t c, const float* const* v_dev, float* const* out_dev) {
   if (!c) return RVE_ERR_ARG;
   if (!v_dev || !out_dev) return bfail(c, RVE_ERR_ARG, "NULL argument");
+  for (int i = 0; i < c->n; ++i)
+    if (!v_dev[i] || !out_dev[i]) return bfail(c, RVE_ERR_ARG, "NULL member field");
+  int dev = 0;
+  BCK(cudaGetDevice(&dev), "device");
+  const bool shared_out = outputs_overlap(c, out_dev);
   MemberFields vin{}, vout{};
   for (int i = 0; i < c->n; ++i) {
-    if (!v_dev[i] || !out_dev[i]) return bfail(c, RVE_ERR_ARG, "NULL member field");
+    const size_t b = (size_t)c->g[i].ncomp * c->g[i].nvox * sizeof(R);
     vin.p[i] = const_cast<R*>(v_dev[i]);
     vout.p[i] = out_dev[i];
+    if (!kernels_reach(v_dev[i], dev)) {
+      vin.p[i] = c->d + c->desc[i].foff;
+      BCK(cudaMemcpyAsync(vin.p[i], v_dev[i], b, cudaMemcpyDeviceToDevice, c->st), "input copy");
+    }
+    if (shared_out || !kernels_reach(out_dev[i], dev)) vout.p[i] = c->Hd + c->desc[i].foff;
   }
   // every input is read (by the x-forward launch) before any output is
   // written (by the x-inverse launch): the fields may alias
@@ -1332,6 +1373,11 @@ rve_status rve_batch_hessp(rve_batch_t c, const float* const* v_dev, float* cons
   BCK(reset_counters(c), "memset");
   BCK(batch_apply(c, nullptr, nullptr, true, nullptr, 0, gate_bits(all), &vin, &vout), "hessp");
   c->hv += c->n;
+  for (int i = 0; i < c->n; ++i) {
+    const size_t b = (size_t)c->g[i].ncomp * c->g[i].nvox * sizeof(R);
+    if (vout.p[i] != out_dev[i])
+      BCK(cudaMemcpyAsync(out_dev[i], vout.p[i], b, cudaMemcpyDeviceToDevice, c->st), "output copy");
+  }
   return RVE_OK;
 }
 

@@ -228,6 +228,7 @@ class RVEBatch:
         self.stream = stream if stream is not None else torch.cuda.current_stream()
         self.shapes = [tuple(reversed(d)) for d in self.dims]
         self.ncomp = [3 if len(d) == 2 else 6 for d in self.dims]
+        self.fshapes = [(nc,) + shp for nc, shp in zip(self.ncomp, self.shapes)]
         self._ids = []
         for ids, shp in zip(phase_ids_list, self.shapes):
             t = torch.as_tensor(ids, dtype=torch.uint8).to(self.device).contiguous()
@@ -251,12 +252,12 @@ class RVEBatch:
             cur.wait_stream(self.stream)
 
     def field(self, i):
-        return torch.empty((self.ncomp[i],) + self.shapes[i], dtype=torch.float32, device=self.device)
+        return torch.empty(self.fshapes[i], dtype=torch.float32, device=self.device)
 
     def hessp(self, vs):
         outs = [self.field(i) for i in range(self.n)]
         for i, v in enumerate(vs):
-            if v.dtype != torch.float32 or tuple(v.shape) != (self.ncomp[i],) + self.shapes[i] or not v.is_contiguous():
+            if v.dtype != torch.float32 or v.shape != self.fshapes[i] or not v.is_contiguous():
                 raise ValueError(f"member {i}: bad field")
         self._in()
         B.rve_batch_hessp(self.h, [v.data_ptr() for v in vs], [o.data_ptr() for o in outs])
