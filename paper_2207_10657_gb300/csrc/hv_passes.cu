@@ -213,6 +213,10 @@ void plan_tiles(const GridDesc& g, SpecWork<R>& w, int wave) {
 template <typename R>
 cudaError_t spectral_plan(const GridDesc& g, SpecWork<R>& w, int wave) {
   plan_tiles<R>(g, w, wave);
+  // a tile that no block can hold is an error here, not a failed launch later
+  // (the sizes that the entry points take all fit)
+  const GenericTiles<R> t(g, w.qx, w.lty, w.ltz, w.px, w.py, w.pz);
+  if (std::max({t.xsmem, t.ysmem, t.zsmem}) > (size_t)kSmemCap) return cudaErrorInvalidValue;
   // opt in to large dynamic shared memory
   cudaFuncSetAttribute(k_xfwd<R, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
   cudaFuncSetAttribute(k_xfwd<R, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);

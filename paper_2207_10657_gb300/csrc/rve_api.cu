@@ -919,10 +919,10 @@ rve_status rve_create(const int dims[3], int ndim, const uint8_t* phase_ids_dev,
     g.nq = nq;
     g.nvox = nq * c->gs.nvox;
     if (ndim == 3) {
-      // the generic passes hold a tile of 36 lines: the x passes one row
-      // (18 packed line pairs of nx points within 16 per thread), the z
-      // pass one column (36 lines of nz points within 24 per thread and the
-      // shared-memory cap)
+      // the generic passes hold a tile of 36 lines: the x passes one row (18
+      // packed line pairs), the z pass one column.  The limits are part of the
+      // interface and inside what a block's shared memory takes, which
+      // spectral_plan checks with the padded lines and tables.
       const size_t csz = (c->opts.precision == 32 ? 8 : 16);
       if (18LL * g.nx > 256LL * 16 || 36LL * g.nz > 512LL * 24 || 36LL * g.nz * csz > 100 * 1024) {
         delete c;
