@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kFT, 4)
   __shared__ __align__(16) float2 buf[NC * Q / 2 * N];
   __shared__ double red[3 * 32];
   const long long row0 = (long long)blockIdx.x * Q;
-  xinv_rows<N, NC, DOT, CG, false>(buf, red, spec, out, dotw, partials, nrows, nxs, nvox, tw, scale, self_dot, cz, cr, cd,
+  xinv_rows<N, NC, DOT, CG>(buf, red, spec, out, dotw, partials, nrows, nxs, nvox, tw, scale, self_dot, cz, cr, cd,
                                    cstatus, calpha, ctau, row0, nrows, blockIdx.x);
 }
 
@@ -140,16 +140,16 @@ __global__ void __launch_bounds__(zthreads<N>(), zminblocks<N>())
 // form, which needs no reordering between the projection and the inverse
 // (256^3: 321 us against 391 us in place).
 template <int N> constexpr bool zinplace() { return N == 384; }
-template <int N> constexpr int zct_tx() { return 4; }  // 75 KB: two blocks per SM
+constexpr int kZipTX = 4;  // columns of a tile: 75 KB, two blocks per SM
 // 256 threads at 128 registers 4241 us per 384^3 product, 512 at 64 registers 4291 us
-template <int N> constexpr int zct_threads() { return 256; }
+constexpr int kZipThreads = 256;
 
 template <int N>
-__global__ void __launch_bounds__(zct_threads<N>(), 2)
+__global__ void __launch_bounds__(kZipThreads, 2)
     kf_zproj_ip(float2* __restrict__ spec, const int ny, const int nxh, const int nxs, const float2* __restrict__ tw,
              const AxisSyms<float> sy, const unsigned free_mask) {
   chain_begin();
-  constexpr int TX = zct_tx<N>(), NT = zct_threads<N>();
+  constexpr int TX = kZipTX, NT = kZipThreads;
   using T = CtTile<N, TX>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* buf = reinterpret_cast<float2*>(smem_raw);
@@ -330,8 +330,8 @@ static cudaError_t ycols_n(const GridDesc& g, float2* spec, const float2* tw, bo
 template <int N>
 static cudaError_t zproj_n(const GridDesc& g, float2* spec, const SpecWork<float>& w, cudaStream_t st) {
   constexpr bool IP = zinplace<N>();
-  constexpr int TX = IP ? zct_tx<N>() : ztx<N>();
-  constexpr int NT = IP ? zct_threads<N>() : zthreads<N>();
+  constexpr int TX = IP ? kZipTX : ztx<N>();
+  constexpr int NT = IP ? kZipThreads : zthreads<N>();
   size_t smem = (size_t)6 * N * TX * sizeof(float2);
   if constexpr (IP) smem = (size_t)6 * CtTile<N, TX>::LP * TX * sizeof(float2);
   auto kernel = [] {

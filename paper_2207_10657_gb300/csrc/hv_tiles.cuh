@@ -250,10 +250,8 @@ __device__ __forceinline__ void xfwd_fft_store(float2* buf, float2* __restrict__
 // r'.r and z'.z per block in partials[3 b + s]; on a boundary or
 // negative-curvature exit, z += tau d.
 // One x-inverse tile: rows [row0, row_end); its block sums go to
-// partials[pidx] (DOT) or partials[3 pidx + s] (CG).  L2LOAD: the spectrum
-// was written by other blocks of the same launch, so it is read through L2
-// (ld.global.cg), never from a stale L1 line.  `red` holds 3 * 32 doubles.
-template <int N, int NC, bool DOT, bool CG, bool L2LOAD>
+// partials[pidx] (DOT) or partials[3 pidx + s] (CG).  `red` holds 3 * 32 doubles.
+template <int N, int NC, bool DOT, bool CG>
 __device__ __forceinline__ void xinv_rows(float2* buf, double* red, const float2* __restrict__ spec,
                                           float* __restrict__ out, const float* __restrict__ dotw,
                                           double* __restrict__ partials, const long long nrows,
@@ -283,8 +281,7 @@ __device__ __forceinline__ void xinv_rows(float2* buf, double* red, const float2
           const int rho = 2 * p + h;
           const int q = rho / NC, c = rho - (rho / NC) * NC;
           const float2* src = spec + c * plane + (row0 + q) * nxs + kk;
-          xh[j][h] = ((JB * GB == NL || p < NL) && row0 + q < row_end) ? (L2LOAD ? __ldcg(src) : *src)
-                                                                       : make_float2(0.f, 0.f);
+          xh[j][h] = (JB * GB == NL || p < NL) && row0 + q < row_end ? *src : make_float2(0.f, 0.f);
         }
       }
 #pragma unroll
@@ -309,7 +306,7 @@ __device__ __forceinline__ void xinv_rows(float2* buf, double* red, const float2
         const int rho = 2 * p + h;
         const int q = rho / NC, c = rho - (rho / NC) * NC;
         const float2* src = spec + c * plane + (row0 + q) * nxs + KB;
-        xn[h] = row0 + q < row_end ? (L2LOAD ? __ldcg(src) : *src) : make_float2(0.f, 0.f);
+        xn[h] = row0 + q < row_end ? *src : make_float2(0.f, 0.f);
       }
       buf[KB * NL + p] = make_float2(xn[0].x, xn[1].x);  // imaginary parts of the Nyquist bin dropped
     }

@@ -72,6 +72,8 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, in
 // shared-memory layout of one CTA (byte offsets; every TMA destination on a
 // 128-byte boundary)
 template <int N> struct TmaLayout {
+  // the scatter and BUF take lines in natural order, N rows of them
+  static_assert(!xinplace<N>(), "the in-place x transform has another layout and more rows");
   static constexpr int Q = xq<N, 6>(), NL = 6 * Q / 2;
   static constexpr int IN = 0;                                       // [6][Q][N] floats
   static constexpr int DMG = IN + 6 * Q * N * 4;                     // [Q][N] floats
