@@ -121,20 +121,35 @@ static void make_plan(int n, AxisPlan& p, bool keep, bool narrow) {
   finish_plan(p);
 }
 
+// Angles from long double libm calls, rounded once to R.  Two calls an entry:
+// on the Grace host long double is software quad arithmetic, and four of them
+// made an FP64 context of 512^2 take 2.8 ms to create instead of 1.9 ms.  FP64
+// wants the half angle too, so it calls for that and doubles it.
+template <typename R>
+void axis_tables(int n, Cx<R>* tw, Cx<R>* gdiff, Cx<R>* gavg) {
+  for (int k = 0; k < n; ++k) {
+    const long double th = 2.0L * 3.14159265358979323846264338327950288L * (long double)k / (long double)n;
+    if constexpr (std::is_same<R, double>::value) {
+      const long double sh = sinl(0.5L * th), ch = cosl(0.5L * th);
+      const long double s = 2.0L * sh * ch, c1 = -2.0L * sh * sh;  // sin th, cos th - 1
+      tw[k] = Cx<R>{(R)(c1 + 1.0L), (R)(-s)};
+      gdiff[k] = (k == 0) ? Cx<R>{0, 0} : Cx<R>{(R)c1, (R)s};
+      gavg[k] = Cx<R>{k == 0 ? (R)0 : (R)sh, 2 * k == n ? (R)0 : (R)ch};
+    } else {
+      const long double c = cosl(th), s = sinl(th);
+      tw[k] = Cx<R>{(R)c, (R)(-s)};
+      gdiff[k] = (k == 0) ? Cx<R>{0, 0} : Cx<R>{(R)(c - 1.0L), (R)s};
+      gavg[k] = (2 * k == n) ? Cx<R>{0, 0} : Cx<R>{(R)((1.0L + c) * 0.5L), (R)(s * 0.5L)};
+    }
+  }
+}
+template void axis_tables<float>(int, float2*, float2*, float2*);
+template void axis_tables<double>(int, double2*, double2*, double2*);
+
 template <typename R>
 static cudaError_t upload_tables(int n, Cx<R>** tw, Cx<R>** gdiff, Cx<R>** gavg) {
   std::vector<Cx<R>> t(n), d(n), a(n);
-  for (int k = 0; k < n; ++k) {
-    // angles from long double libm calls, rounded once to R
-    const long double th = 2.0L * 3.14159265358979323846264338327950288L * (long double)k / (long double)n;
-    const long double c = cosl(th), s = sinl(th);
-    t[k] = Cx<R>{(R)c, (R)(-s)};
-    d[k] = (k == 0) ? Cx<R>{0, 0} : Cx<R>{(R)(c - 1.0L), (R)s};
-    if (std::is_same<R, double>::value)
-      a[k] = Cx<R>{k == 0 ? (R)0 : (R)sinl(0.5L * th), 2 * k == n ? (R)0 : (R)cosl(0.5L * th)};
-    else
-      a[k] = (2 * k == n) ? Cx<R>{0, 0} : Cx<R>{(R)((1.0L + c) * 0.5L), (R)(s * 0.5L)};
-  }
+  axis_tables<R>(n, t.data(), d.data(), a.data());
   cudaError_t e;
   if ((e = cudaMalloc(tw, n * sizeof(Cx<R>))) != cudaSuccess) return e;
   if ((e = cudaMalloc(gdiff, n * sizeof(Cx<R>))) != cudaSuccess) return e;

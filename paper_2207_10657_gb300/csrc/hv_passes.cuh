@@ -109,6 +109,10 @@ template <typename R> struct GenericTiles {
   GenericTiles(const GridDesc& g, int qx, int lty, int ltz, const AxisPlan& px, const AxisPlan& py,
                const AxisPlan& pz);
 };
+// Twiddles and gradient factors of an axis of n points (the host arrays of
+// SpecWork's tw, gdiff and gavg).
+template <typename R>
+void axis_tables(int n, Cx<R>* tw, Cx<R>* gdiff, Cx<R>* gavg);
 // Stage tables of a plan from its radices.
 void finish_plan(AxisPlan& p);
 
