@@ -76,9 +76,9 @@ template <int N> constexpr size_t cl_smem() {
 template <int N, int MODE>
 __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kFT, 2)
     kc_xyfwd(const float* __restrict__ in, const uint8_t* __restrict__ phase, const float* __restrict__ dmg,
-             const MatTable<float> mt, float2* __restrict__ spec, const int nz, const int nxs, const long long nvox,
+             const MatTable<float> mt, float2* __restrict__ spec, const int nz, const long long nvox,
              const float2* __restrict__ twn, const float2* __restrict__ twm, double* __restrict__ partials) {
-  constexpr int M = N / kCR, NXH = N / 2 + 1, LY = NXH;
+  constexpr int M = N / kCR, NXH = N / 2 + 1, LY = NXH, NXS = spectrum_stride(NXH);
   constexpr int NLB = cl_nlb<N>(), BR = 2 * NLB, NBT = M / BR;
   constexpr int NLW = NLB + 1;  // odd line stride of the x batch: consecutive x on distinct banks
   constexpr int K2 = M / kCR;  // frequencies k2 finished by each CTA
@@ -160,7 +160,7 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kFT, 2)
   unsigned rb[kCR];
 #pragma unroll
   for (int q = 0; q < kCR; ++q) rb[q] = cl_map(yb, q);
-  float2* out = spec + ((long long)c * nz + z) * N * nxs;
+  float2* out = spec + ((long long)c * nz + z) * N * NXS;
   for (int it = threadIdx.x; it < K2 * NXH; it += kFT) {
     const int k2 = r * K2 + it / NXH, kx = it - (it / NXH) * NXH;
     const unsigned off = (unsigned)(k2 * LY + kx) * (unsigned)sizeof(float2);
@@ -171,7 +171,7 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kFT, 2)
     for (int q = 1; q < kCR; ++q) a[q] = cmul(a[q], __ldg(&twn[q * k2]));
     Dft<kCR, false, float2>::run(a);
 #pragma unroll
-    for (int k1 = 0; k1 < kCR; ++k1) out[(long long)(k2 + M * k1) * nxs + kx] = a[k1];
+    for (int k1 = 0; k1 < kCR; ++k1) out[(long long)(k2 + M * k1) * NXS + kx] = a[k1];
   }
   // no CTA leaves while the others may still read its Y
   cl_sync();
@@ -190,11 +190,11 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kFT, 2)
 template <int N, bool DOT, bool CG>
 __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kFT, 2)
     kc_yxinv(const float2* __restrict__ spec, float* __restrict__ out, const float* __restrict__ dotw,
-             double* __restrict__ partials, const int nz, const int nxs, const long long nvox, const float2* __restrict__ twn,
+             double* __restrict__ partials, const int nz, const long long nvox, const float2* __restrict__ twn,
              const float2* __restrict__ twm, const float scale, const bool self_dot, float* __restrict__ cz,
              float* __restrict__ cr, const float* __restrict__ cd, const int* __restrict__ cstatus,
              const double* __restrict__ calpha, const double* __restrict__ ctau) {
-  constexpr int M = N / kCR, NXH = N / 2 + 1, LY = NXH;
+  constexpr int M = N / kCR, NXH = N / 2 + 1, LY = NXH, NXS = spectrum_stride(NXH);
   constexpr int NLB = cl_nlb<N>(), BR = 2 * NLB, NBT = M / BR;
   constexpr int NLW = NLB + 1;  // odd line stride of the x batch: consecutive x on distinct banks
   constexpr int K2 = M / kCR;
@@ -210,12 +210,12 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kFT, 2)
   unsigned rb[kCR];
 #pragma unroll
   for (int q = 0; q < kCR; ++q) rb[q] = cl_map(yb, q);
-  const float2* src = spec + ((long long)c * nz + z) * N * nxs;
+  const float2* src = spec + ((long long)c * nz + z) * N * NXS;
   for (int it = threadIdx.x; it < K2 * NXH; it += kFT) {
     const int k2 = r * K2 + it / NXH, kx = it - (it / NXH) * NXH;
     float2 a[kCR];
 #pragma unroll
-    for (int k1 = 0; k1 < kCR; ++k1) a[k1] = src[(long long)(k2 + M * k1) * nxs + kx];
+    for (int k1 = 0; k1 < kCR; ++k1) a[k1] = src[(long long)(k2 + M * k1) * NXS + kx];
     Dft<kCR, true, float2>::run(a);
 #pragma unroll
     for (int q = 1; q < kCR; ++q) a[q] = cmulc(a[q], __ldg(&twn[q * k2]));
@@ -324,6 +324,7 @@ __global__ void __cluster_dims__(kCR, 1, 1) __launch_bounds__(kFT, 2)
 // ================================================================ host side
 bool cluster_size_ok(const GridDesc& g) {
   if (g.ndim != 3 || g.nq != 1 || g.ncomp != 6 || g.nx != g.ny) return false;
+  if (g.nxs != spectrum_stride(g.nxh)) return false;  // the kernels' row stride is a constant
   return g.nx == 64 || g.nx == 128 || g.nx == 256 || g.nx == 96 || g.nx == 192;
 }
 
@@ -352,10 +353,10 @@ static cudaError_t xyfwd_n(const GridDesc& g, const float* in, const uint8_t* ph
   cudaError_t e;
   if (tangent) {
     if ((e = cl_attr<kc_xyfwd<N, 1>>(sm)) != cudaSuccess) return e;
-    kc_xyfwd<N, 1><<<blocks, kFT, sm, st>>>(in, phase, dmg, mt, spec, g.nz, g.nxs, g.nvox, twn, twm, partials);
+    kc_xyfwd<N, 1><<<blocks, kFT, sm, st>>>(in, phase, dmg, mt, spec, g.nz, g.nvox, twn, twm, partials);
   } else {
     if ((e = cl_attr<kc_xyfwd<N, 0>>(sm)) != cudaSuccess) return e;
-    kc_xyfwd<N, 0><<<blocks, kFT, sm, st>>>(in, phase, dmg, mt, spec, g.nz, g.nxs, g.nvox, twn, twm, nullptr);
+    kc_xyfwd<N, 0><<<blocks, kFT, sm, st>>>(in, phase, dmg, mt, spec, g.nz, g.nvox, twn, twm, nullptr);
   }
   return cudaGetLastError();
 }
@@ -369,7 +370,7 @@ static cudaError_t yxinv_launch(const GridDesc& g, const float2* spec, float* ou
   cudaError_t e;
   if ((e = cl_attr<kc_yxinv<N, DOT, CG>>(sm)) != cudaSuccess) return e;
   const float scale = (float)(1.0 / (double)g.nvox);
-  kc_yxinv<N, DOT, CG><<<cluster_blocks(g), kFT, sm, st>>>(spec, out, dotw, partials, g.nz, g.nxs, g.nvox, twn, twm, scale,
+  kc_yxinv<N, DOT, CG><<<cluster_blocks(g), kFT, sm, st>>>(spec, out, dotw, partials, g.nz, g.nvox, twn, twm, scale,
                                                            self, z, r, d, status, alpha, tau);
   return cudaGetLastError();
 }

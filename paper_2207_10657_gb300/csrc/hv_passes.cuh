@@ -26,7 +26,7 @@ struct GridDesc {
 // straddles five sectors instead of four (product at 128^3 161.6 -> 159.8 us, 64^3
 // 43.0 -> 41.2 us; 128-byte rows instead: 256^3 1046 -> 1084 us).  Not for rows
 // shorter than that pays (32^3: 28.7 us as they are, 30.7 us padded).
-inline int spectrum_stride(int nxh) { return nxh <= 24 ? nxh : (nxh + 3) & ~3; }
+__host__ __device__ constexpr int spectrum_stride(int nxh) { return nxh <= 24 ? nxh : (nxh + 3) & ~3; }
 
 // Rank-one part of the symmetric consistent damage tangent, per voxel: the
 // tangent applied to v is (1-D) C : v - dp/2 (a (n.v) + n (a.v)) with
