@@ -3,10 +3,10 @@
 // into immediates.  The radix sequence is that of fft_radix (8, 4, 4, 3), the
 // last two taken in registers one after the other.
 //
-// It was tried for every compiled length.  Wider pairs (256 = 8 x 32, two
-// trips through shared memory) take 90-128 registers and lose more to the
-// missing warps than they save: z pass 420 us against 327 us, y pass 180 us
-// against 150 us at 256^3; single radices 391 and 150 us.
+// Tried at 256^3 as well: wider pairs (256 = 8 x 32, two trips through shared
+// memory) take 90-128 registers and lose more to the missing warps than they
+// save: z pass 420 us against 327 us, y pass 180 us against 150 us; single
+// radices 391 and 150 us.
 #pragma once
 
 #include "fft_fast.cuh"

@@ -1,10 +1,10 @@
 // In-place mixed-radix FFT of lines held in shared memory, lengths and
 // radices known at run time: the engine of the generic passes (FP64 fields,
 // lengths without compiled passes, the batched solver, Kuhn tetrahedra).
-// Products on it, self-sorting form before -> now: FP32 160x120x90 638 -> 222
-// us; FP64 128^3 2981 -> 1958 us, 84 % of the FP64 pipe's rate in the y
-// passes; Kuhn tetrahedra 64^3 380 -> 227 us; 96 uneven cells, the passes
-// alone 6.3 -> 3.0 ms.  (The x passes' tables of XTables came after these figures.)
+// Products, with the self-sorting form it replaced -> with it and with what the
+// passes gained since (tables of the x tiles, padded rows, chained launches):
+// FP32 160x120x90 638 -> 187 us; FP64 128^3 2981 -> 1865 us; Kuhn tetrahedra
+// 64^3 380 -> 176 us.  By itself it took them to 222, 1958 and 227 us.
 //
 // A line of n = r_0 r_1 ... r_{S-1} elements is a mixed-radix number: element
 // x = d_0 m_0 + d_1 m_1 + ... with m_s = n / (r_0 ... r_s).  Stage s replaces

@@ -184,17 +184,23 @@ template struct GenericTiles<double>;
 // Such a grid leaves most SMs a warp or two, and an FP64 instruction occupies
 // its scheduler for 64 cycles however few lanes it has: a stage's time is the
 // number of instructions of ONE butterfly, so small butterflies spread over
-// more warps win.  Products, wide -> narrow: 16^2 33.7 -> 22.1 us, 60x90 46.5 ->
-// 38.4, 128^2 (49152 values) 53.8 -> 37.7, 16^3 51.8 -> 35.3; past the line
-// the pipe is full and the extra trips through shared memory lose: 256^2 and
-// 32^3 (196608 values) 52.3 -> 62.6 and 62.3 -> 67.3.
+// more warps win.  Products, wide -> narrow: 16^2 33.6 -> 21.9 us, 90x60 50.1 ->
+// 40.3, 128^2 (49152 values) 53.9 -> 37.7, 16^3 51.9 -> 35.5.  Once the pipe is
+// full the extra trips through shared memory lose: 192^2 (110592 values) 48.5
+// -> 59.4, 256^2 52.3 -> 62.6, 32^3 62.6 -> 67.3.  Around the line the lengths
+// decide: 144x150 (64800) 50.1 -> 51.9, 18x20x30 (64800) 55.0 -> 47.5, 150^2
+// (67500) 44.5 -> 52.6, 24x24x20 (69120) 76.0 -> 54.0, 160^2 73.6 -> 46.8, 24^3
+// (82944) 56.0 -> 58.9.
 constexpr long long kNarrowMax = 65536;
 
 // Plans and tiles.  A tile is as large as keeps its threads busy (about one
 // butterfly each, 128-byte column segments) and as small as gives the grid
 // `wave` blocks, which alone on the chip leaves every SM work: with one tile size for all grids, each pass of a 32^2 cell ran on ONE
-// SM (FP64 product 129 -> 35 us with 16-17 blocks per pass).  Columns do not
-// go below the 32 bytes of a memory sector while a tile fits a block.
+// SM (FP64 product 129 -> 35 us with 16-17 blocks per pass).  The element
+// budgets leave the 32 bytes of a memory sector to a tile's columns; three
+// limits go below that: what fits a block, the blocks wanted of a small grid,
+// and the frequencies a block can hold while an FP32 tile is reordered (kHold:
+// two columns at z lengths above 256, one above 512).
 template <typename R>
 void plan_tiles(const GridDesc& g, SpecWork<R>& w, int wave) {
   using C = Cx<R>;

@@ -24,8 +24,11 @@ struct GridDesc {
 // FP64), so that the column segments of the y and z passes touch no sector in
 // vain; nx/2 + 1 itself is odd for most lengths, and a 128-byte segment then
 // straddles five sectors instead of four (product at 128^3 161.6 -> 159.8 us, 64^3
-// 43.0 -> 41.2 us; 128-byte rows instead: 256^3 1046 -> 1084 us).  Not for rows
-// shorter than that pays (32^3: 28.7 us as they are, 30.7 us padded).
+// 43.0 -> 41.2 us; 128-byte rows instead: 256^3 1046 -> 1084 us).  Short rows
+// stay as they are: the padding is a larger part of them, and such grids are
+// small (products, as they are / padded: 36x32x32 (19 values a row) 18.0 / 18.8
+// us, 40x64x64 (21) 29.0 / 28.2; 48x64x64 (25) 29.5 / 28.7, 54x64x64 (28) 28.7 /
+// 28.7).
 __host__ __device__ constexpr int spectrum_stride(int nxh) { return nxh <= 24 ? nxh : (nxh + 3) & ~3; }
 
 // Rank-one part of the symmetric consistent damage tangent, per voxel: the

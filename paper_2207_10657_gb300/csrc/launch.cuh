@@ -23,7 +23,9 @@ namespace rve {
 __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Launch a kernel that starts with chain_begin().  Under stream capture the
-// launch is an ordinary one: captured graphs keep full kernel dependencies.
+// launch is an ordinary one: captured graphs (the CG loop's conditional body
+// among them) keep full kernel dependencies.  What programmatic edges would
+// give there has not been measured.
 template <typename... P, typename... A>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
