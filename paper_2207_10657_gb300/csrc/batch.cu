@@ -33,7 +33,8 @@ using C = float2;
 constexpr int kMaxBatch = 256;
 // resident blocks per SM of the x / y / 2D launches: the items' starts are
 // latency, so two more blocks than the single-grid kernels pay here (96 cells
-// 2.87 -> 2.70 ms; a single 160x120x90 grid 199 -> 206 us)
+// 2.42 -> 2.21 ms, 8 cells of 512^2 160 -> 140 us; a single 160x120x90 grid 199 ->
+// 206 us)
 constexpr int kXYPerSM = 8;
 // Items that a batched launch should have at least, shared out over the
 // members of one dimension by their field values: a member's tiles shrink only

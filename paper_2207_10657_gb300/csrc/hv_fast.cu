@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kFT)
 }
 
 // The in-place form, for the length whose Stockham tile takes ten columns (80
-// of the 128 bytes of a segment): 16 columns, 606 -> 471 us per pass at 384^3.
+// of the 128 bytes of a segment): 16 columns, 606 -> 481 us per pass at 384^3.
 template <int N> constexpr bool yinplace() { return N == 384; }
 
 template <int N, bool INV>
